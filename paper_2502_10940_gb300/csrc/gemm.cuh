@@ -1143,8 +1143,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                             bulk_commit_group();
                         }
                         out_slot = 0;
-                    } else {
-                        if (c0 < nch) put(p, map_d, p.d_ptr, wsave[i], n_blk * BN + c0 * 32, row0, row);
+                    } else if (c0 < nch) {
+                        // emit waits for all but the newest group, but the newest
+                        // one may be a pair that still reads both boxes
+                        if (lane == 0) bulk_wait_group_read<0>();
+                        put(p, map_d, p.d_ptr, wsave[i], n_blk * BN + c0 * 32, row0, row);
                         if (c1 < nch) put(p, map_d, p.d_ptr, wsave[i + 1], n_blk * BN + c1 * 32, row0, row);
                     }
                 }
