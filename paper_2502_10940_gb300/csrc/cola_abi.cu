@@ -835,29 +835,41 @@ cola_status_t run_glu(const Shape& s, const void* H_cat, int64_t ldh, const void
     return launched(traced(COLA_KERNEL_FWD_GLU, 1, mnk, 1, flags, st, [&] { return dispatch_glu(bn, pair, b, sms, st); }));
 }
 
+// From this K on the gated dX GEMM takes the epilogue that leaves a deeper
+// operand ring (EPI_GLU_BWD_LONG).  Measured two-box against one-box slots:
+// K = 512 583 / 635 us (65536 x 5461), K = 1024 830 / 680 us (32768 x 11008).
+constexpr int64_t GLU_LONG_K = 768;
+
 // The down layer's input gradient when its input is M = Y_gate * Y_up: the
 // dX GEMM dM = dZ A (dZ [n x K] pitch ldz) whose epilogue stores
 // dY_gate = bf16(dM) * Y_up and dY_up = bf16(dM) * Y_gate (all pitch ld_x).
 cola_status_t run_b4_glu(const Shape& s, int64_t K, const void* dZ, int64_t ldz, const void* A, const void* Yg,
                          const void* Yu, void* dYg, void* dYu, unsigned int* status, int sms, cudaStream_t st)
 {
-    const int bn = choose_bn_for(s.n, s.d_in, K);
-    const int ms = choose_msub(s.n, s.d_in, K, bn);
+    // CTA pairs where the plain dX GEMM takes them; otherwise 128 x 128 tiles
+    // (256-column ones would leave two operand stages beside the slots of
+    // Y_gate and Y_up boxes)
+    const int bn_x = choose_bn_for(s.n, s.d_in, K);
+    const bool pair = choose_msub(s.n, s.d_in, K, bn_x) == TILE_PAIR;
+    const int bn = pair ? 256 : 128;
+    const int ms = pair ? TILE_PAIR : 1;
     GemmProblem pr;
     std::memset(&pr, 0, sizeof pr);
     pr.p = base_params(s.n, s.d_in, K, bn, ms);
     COLA_MAP(map_kmajor(&pr.map_a, dZ, K, s.n, ldz, a_box_rows(ms)));
     COLA_MAP(map_mnmajor(&pr.map_b, A, s.d_in, K, s.ld_a));
-    COLA_MAP(map_box32(&pr.map_d, dYg, s.d_in, s.n, s.ld_x));
-    COLA_MAP(map_box32(&pr.map_d2, dYu, s.d_in, s.n, s.ld_x));
-    pr.map_z = pr.map_d3 = pr.map_b2 = pr.map_d;
+    COLA_MAP(map_box64(&pr.map_d, dYg, s.d_in, s.n, s.ld_x));
+    COLA_MAP(map_box64(&pr.map_d2, dYu, s.d_in, s.n, s.ld_x));
+    COLA_MAP(map_box64(&pr.map_z, Yg, s.d_in, s.n, s.ld_x));
+    COLA_MAP(map_box64(&pr.map_d3, Yu, s.d_in, s.n, s.ld_x));
+    pr.map_b2 = pr.map_d;
     pr.p.d_ptr = static_cast<__nv_bfloat16*>(dYg);
     pr.p.d2_ptr = static_cast<__nv_bfloat16*>(dYu);
     pr.p.d_ld = s.ld_x;
-    pr.p.yg_ptr = static_cast<const __nv_bfloat16*>(Yg);
-    pr.p.yu_ptr = static_cast<const __nv_bfloat16*>(Yu);
     pr.p.status = status;
     const int64_t mnk[1][3] = {{s.n, s.d_in, K}};
+    if (pair && K >= GLU_LONG_K)
+        return run_batch<false, true, EPI_GLU_BWD_LONG>(COLA_KERNEL_BWD_DX, bn, ms, &pr, mnk, 1, TRACE_GLU, sms, st);
     return run_batch<false, true, EPI_GLU_BWD>(COLA_KERNEL_BWD_DX, bn, ms, &pr, mnk, 1, TRACE_GLU, sms, st);
 }
 
@@ -865,8 +877,13 @@ cola_status_t run_b4_glu(const Shape& s, int64_t K, const void* dZ, int64_t ldz,
 cola_status_t run_b4(const Shape& s, int64_t K, const void* dZ, int64_t ldz, const void* A, void* dX,
                      unsigned int* status, int sms, cudaStream_t st)
 {
-    const int bn = choose_bn_for(s.n, s.d_in, K);
-    const int ms = choose_msub(s.n, s.d_in, K, bn);
+    // CTA pairs where the plain dX GEMM takes them; otherwise 128 x 128 tiles
+    // (256-column ones would leave two operand stages beside the slots of
+    // Y_gate and Y_up boxes)
+    const int bn_x = choose_bn_for(s.n, s.d_in, K);
+    const bool pair = choose_msub(s.n, s.d_in, K, bn_x) == TILE_PAIR;
+    const int bn = pair ? 256 : 128;
+    const int ms = pair ? TILE_PAIR : 1;
     GemmProblem pr;
     std::memset(&pr, 0, sizeof pr);
     pr.p = base_params(s.n, s.d_in, K, bn, ms);

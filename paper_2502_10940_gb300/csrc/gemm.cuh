@@ -44,9 +44,10 @@
 //               and the up half H_up B_up^T into a second accumulator of the
 //               same tile, and the epilogue stores M = bf16(Y_gate * Y_up) of
 //               the bf16-rounded outputs (and Y_gate, Y_up when training)
-//   EPI_GLU_BWD dX GEMM of the down layer whose input is that M: with
-//               dM = bf16(acc) it stores dY_gate = bf16(dM * Y_up) and
-//               dY_up = bf16(dM * Y_gate), reading Y_gate, Y_up per chunk
+//   EPI_GLU_BWD (and _LONG, for long K walks) dX GEMM of the down layer whose
+//               input is that M: with dM = bf16(acc) it stores
+//               dY_gate = bf16(dM * Y_up) and dY_up = bf16(dM * Y_gate) over
+//               TMA-loaded boxes of Y_up and Y_gate
 //   EPI_TAIL      weight gradients (bf16 D) with a split tail: the tiles of
 //               the full waves run whole and store D = bf16(acc) as
 //               EPI_STORE; the tiles of the last, partial wave are split
@@ -94,7 +95,7 @@ enum : unsigned int {
 
 enum Epi : int {
     EPI_STORE = 0, EPI_ZH = 1, EPI_DSIGMA = 2, EPI_F32 = 3, EPI_TAIL = 4, EPI_GLU = 5, EPI_GLU_BWD = 6,
-    EPI_DSIGMA_H = 7
+    EPI_DSIGMA_H = 7, EPI_GLU_BWD_LONG = 8
 };
 enum Sigma : int { SIG_IDENTITY = 0, SIG_SILU = 1, SIG_GELU = 2 };
 
@@ -122,14 +123,11 @@ struct GemmParams {
     long long d_ld;
     int sigma;
     unsigned int* status;
-    // gated MLP (EPI_GLU, EPI_GLU_BWD): the outputs behind map_d2 and map_d3,
-    // for the masked stores of a ragged right edge (pitch d_ld), and the
-    // Y_gate, Y_up that the EPI_GLU_BWD epilogue reads (pitch d_ld)
+    // gated MLP: the outputs behind map_d2 (EPI_GLU, EPI_GLU_BWD) and map_d3
+    // (EPI_GLU), for the masked stores of a ragged right edge (pitch d_ld)
     int glu_half;                 // EPI_GLU: k-blocks of the gate half; the up half reads map_b2
     __nv_bfloat16* d2_ptr;
     __nv_bfloat16* d3_ptr;
-    const __nv_bfloat16* yg_ptr;
-    const __nv_bfloat16* yu_ptr;
     // problem 0 only, for the failure-detection self-tests: 1 = the producers
     // issue nothing, so the MMA's first wait runs out; 2 = the odd CTA of a
     // pair issues its first k-block only, so the MMA's second wait runs out
@@ -138,8 +136,8 @@ struct GemmParams {
 };
 
 // Epilogue staging: per epilogue warp two 2 KB boxes of 32 rows x 32 bf16
-// columns (64-byte rows, 64-byte TMA swizzle).  EPI_STORE / EPI_ZH / EPI_GLU /
-// EPI_GLU_BWD use them as a ring of output boxes.  EPI_DSIGMA uses them as a double buffer for the
+// columns (64-byte rows, 64-byte TMA swizzle).  EPI_STORE / EPI_ZH / EPI_GLU
+// use them as a ring of output boxes.  EPI_DSIGMA uses them as a double buffer for the
 // saved Z: the box of the warp's next chunk is TMA-loaded while the current
 // one is processed, and dZ is computed in place and TMA-stored from the box.
 constexpr int EPI_BOX_BYTES = 32 * 32 * 2;
@@ -147,6 +145,33 @@ constexpr int EPI_OUT_BOXES = 2;
 static_assert(EPI_OUT_BOXES == 2, "the CTA-pair store epilogue stages a chunk pair into the whole ring");
 constexpr int EPI_WARP_BYTES = EPI_OUT_BOXES * EPI_BOX_BYTES;
 constexpr int EPI_SMEM_BYTES = NUM_EPI_WARPS * EPI_WARP_BYTES;
+// The gated dX epilogue works on chunks of 64 columns: a box of 32 rows
+// (128-byte rows, 128-byte swizzle) of Y_up and one of Y_gate, TMA-loaded
+// ahead of their use; each gradient is computed in place and TMA-stored from
+// the same box.  Its launch moves four d_ff-wide tensors for one short K walk,
+// so it is bound by HBM and by what the TMA engine of an SM sustains beside
+// the operand loads.
+//   EPI_GLU_BWD       two slots of both boxes per warp (16 KB), one chunk
+//                     ahead; leaves 3 operand stages (128 x 128 per CTA and
+//                     k-block).  65536 x 5461, K = 512: 955 -> 583 us;
+//                     65536 x 2736, K = 256: 228 us (6.3 TB/s).
+//   EPI_GLU_BWD_LONG  a ring of three single boxes per warp (12 KB), two ahead;
+//                     4 operand stages, for K walks long enough to be held up
+//                     by the operand ring.  32768 x 11008, K = 1024: 768 ->
+//                     680 us (two-box slots: 830 us; at K = 512 635 us).
+// The former epilogue loaded Y_gate and Y_up from global memory by rows.  Boxes
+// of 32 columns (64-byte rows): 714 us at K = 512 (5461-element rows are not
+// 32-byte aligned: more TMA requests and partial sectors); 16 warps of one
+// chunk each: 630 us; 128-column pair tiles: 702 us.
+constexpr int GLU_COLS = 64;
+constexpr int GLU_BOX_BYTES = 32 * GLU_COLS * 2;
+constexpr bool epi_glu_bwd(int epi) { return epi == EPI_GLU_BWD || epi == EPI_GLU_BWD_LONG; }
+constexpr int epi_slots(int epi) { return epi == EPI_GLU_BWD_LONG ? 3 : 2; }   // side-input slots per warp
+constexpr int epi_slot_bytes(int epi)
+{
+    return epi == EPI_GLU_BWD ? 2 * GLU_BOX_BYTES : epi == EPI_GLU_BWD_LONG ? GLU_BOX_BYTES : EPI_BOX_BYTES;
+}
+constexpr int epi_warp_bytes(int epi) { return epi_glu_bwd(epi) ? epi_slots(epi) * epi_slot_bytes(epi) : EPI_WARP_BYTES; }
 
 // A CTA tile is MSUB x 128 rows by BN columns: MSUB = 2 runs two M = 128
 // MMAs per k-step that share one B tile (halving the B-operand traffic per
@@ -154,7 +179,8 @@ constexpr int EPI_SMEM_BYTES = NUM_EPI_WARPS * EPI_WARP_BYTES;
 // 128-row tile with two accumulators (the gate and up halves of EPI_GLU).
 // BUFS: tiles whose accumulators TMEM holds at once (2: the epilogue of one
 // tile overlaps the main loop of the next).
-template <int BN, int MSUB, bool PAIR = false, int ACCS = 1, int BUFS = 2>
+// EPI_BYTES: epilogue staging of all warps.
+template <int BN, int MSUB, bool PAIR = false, int ACCS = 1, int BUFS = 2, int EPI_BYTES = EPI_SMEM_BYTES>
 struct GemmCfg {
     static_assert(BN % 64 == 0 && BN >= 64 && BN <= 256, "BN must be 64..256 in steps of 64");
     static_assert(MSUB == 1 || MSUB == 2, "one or two 128-row sub-tiles");
@@ -167,14 +193,20 @@ struct GemmCfg {
     static constexpr int A_BYTES = CTA_ROWS * BK * 2;
     static constexpr int B_BYTES = B_ROWS * BK * 2;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int BAR_BYTES = 512;        // 39 mbarriers, the TMEM address, the abort flag, a count
+    static constexpr int BAR_BYTES = 512;        // <= 47 mbarriers, the TMEM address, the abort flag, a count
     static constexpr int SMEM_LIMIT = 232448;   // opt-in maximum per CTA
-    static constexpr int STAGES_FIT = (SMEM_LIMIT - 1024 - BAR_BYTES - EPI_SMEM_BYTES) / STAGE_BYTES;
+    static constexpr int STAGES_FIT = (SMEM_LIMIT - 1024 - BAR_BYTES - EPI_BYTES) / STAGE_BYTES;
     static constexpr int STAGES = STAGES_FIT > 8 ? 8 : STAGES_FIT;
     static constexpr int TMEM_COLS = (BUFS * ACC_COLS <= 128) ? 128 : (BUFS * ACC_COLS <= 256 ? 256 : 512);
-    static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + EPI_SMEM_BYTES + BAR_BYTES;
+    static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + EPI_BYTES + BAR_BYTES;
     static_assert(SMEM_BYTES <= SMEM_LIMIT, "shared memory budget");
 };
+
+// The configuration of a kernel whose epilogue is EPI: EPI_GLU holds a gate
+// and an up accumulator per tile (one tile at a time with 256 columns).
+template <int BN, int MSUB, bool PAIR, int EPI>
+using EpiGemmCfg = GemmCfg<BN, MSUB, PAIR, EPI == EPI_GLU ? 2 : 1, (EPI == EPI_GLU && BN == 256) ? 1 : 2,
+                           NUM_EPI_WARPS * epi_warp_bytes(EPI)>;
 
 // two bf16 values packed in a 32-bit word (low half first) and back
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
@@ -185,6 +217,14 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
+
+// The bf16 products of two packed pairs, each rounded once.
+__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b)
+{
+    const __nv_bfloat162 v =
+        __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
 
 // ------------------------------------------------------------ activations
 // The logistic s(z) = 1 / (1 + e^{-z}) of SiLU, in two forms:
@@ -451,7 +491,7 @@ constexpr int MAX_GROUP = 4;
 // One GEMM of a batch: its operand / output tensor maps and parameters.
 struct GemmProblem {
     CUtensorMap map_a, map_b, map_d, map_d2, map_z;
-    CUtensorMap map_b2, map_d3;   // EPI_GLU: B_up, and the Y_up output
+    CUtensorMap map_b2, map_d3;   // EPI_GLU: B_up, and the Y_up output; EPI_GLU_BWD: map_z Y_gate, map_d3 Y_up
     GemmParams p;
     int unit_begin;   // first batch-wide unit index of this problem
 };
@@ -568,6 +608,20 @@ __device__ __forceinline__ void stage_row(uint32_t box, int lane, const uint32_t
     for (int j = 0; j < 4; ++j) st_shared_v4(box + box64_off(lane, j), w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
 }
 
+// Store the first `valid` (up to 8) of 8 packed bf16 at d (16-byte aligned).
+__device__ __forceinline__ void store_row8(__nv_bfloat16* d, const uint4& w, int valid)
+{
+    if (valid >= 8) {
+        *reinterpret_cast<uint4*>(d) = w;
+        return;
+    }
+    const uint32_t v[4] = {w.x, w.y, w.z, w.w};
+    uint16_t* d16 = reinterpret_cast<uint16_t*>(d);
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        if (e < valid) d16[e] = static_cast<uint16_t>((e & 1) ? (v[e >> 1] >> 16) : (v[e >> 1] & 0xFFFFu));
+}
+
 // ------------------------------------------------------------ the kernel
 template <int BN, int MSUB, bool A_MN, bool B_MN, int EPI, bool PAIR = false, int SIG = SIG_IDENTITY>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
@@ -592,22 +646,27 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     // a run-time switch between the two made the LLaMA-60M dZ GEMMs 4-10 %
     // slower)
     constexpr bool DSIG = EPI == EPI_DSIGMA || EPI == EPI_DSIGMA_H;
-    using C = GemmCfg<BN, MSUB, PAIR, EPI == EPI_GLU ? 2 : 1, GLU_SPLIT ? 1 : 2>;
+    using C = EpiGemmCfg<BN, MSUB, PAIR, EPI>;
+    constexpr bool GLU_BWD = epi_glu_bwd(EPI);
+    constexpr bool GLU_ONE = EPI == EPI_GLU_BWD_LONG;   // one box per slot
+    constexpr int WARP_BYTES = epi_warp_bytes(EPI);
+    constexpr int ZSLOTS = epi_slots(EPI);          // side-input slots per epilogue warp
+    constexpr int CHUNK = GLU_BWD ? GLU_COLS : 32;      // columns of one epilogue chunk
     constexpr int STAGES = C::STAGES;
     constexpr int TILE_M = C::TILE_M;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* smem_a = smem;                              // STAGES x A_BYTES
     uint8_t* smem_b = smem + STAGES * C::A_BYTES;        // STAGES x B_BYTES
-    uint8_t* smem_epi = smem + STAGES * C::STAGE_BYTES;  // NUM_EPI_WARPS x EPI_WARP_BYTES
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem_epi + EPI_SMEM_BYTES);
+    uint8_t* smem_epi = smem + STAGES * C::STAGE_BYTES;  // NUM_EPI_WARPS x WARP_BYTES
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem_epi + NUM_EPI_WARPS * WARP_BYTES);
     uint64_t* full_bar = bars;                 // [STAGES]
     uint64_t* empty_bar = bars + STAGES;       // [STAGES]
     uint64_t* tfull_bar = bars + 2 * STAGES;   // [2]
     uint64_t* tempty_bar = tfull_bar + 2;      // [2]
     uint64_t* drain_bar = tempty_bar + 2;      // [1]
-    uint64_t* zfull_bar = drain_bar + 1;       // [NUM_EPI_WARPS][2]  Z boxes (EPI_DSIGMA)
-    uint64_t* xchg_bar = zfull_bar + 2 * NUM_EPI_WARPS;   // [1] PAIR: the odd producer's report (even CTA)
+    uint64_t* zfull_bar = drain_bar + 1;       // [NUM_EPI_WARPS][ZSLOTS]  Z (EPI_DSIGMA), Y_gate and Y_up (EPI_GLU_BWD)
+    uint64_t* xchg_bar = zfull_bar + ZSLOTS * NUM_EPI_WARPS;   // [1] PAIR: the odd producer's report (even CTA)
     uint64_t* relay_bar = xchg_bar + 1;        // [1] PAIR: the even CTA's drain is done (odd CTA)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(relay_bar + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -633,7 +692,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             mbar_init(&tempty_bar[b], NUM_EPI_WARPS * 32 * (PAIR ? 2 : 1));   // PAIR: both CTAs' epilogues
         }
         mbar_init(drain_bar, 1);
-        for (int j = 0; j < 2 * NUM_EPI_WARPS; ++j) mbar_init(&zfull_bar[j], 1);
+        for (int j = 0; j < ZSLOTS * NUM_EPI_WARPS; ++j) mbar_init(&zfull_bar[j], 1);
         mbar_init(xchg_bar, 1);
         mbar_init(relay_bar, 1);
         *abort_flag = 0;
@@ -643,7 +702,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             tma_prefetch_desc(&batch.prob[g].map_a);
             tma_prefetch_desc(&batch.prob[g].map_b);
             if (EPI != EPI_F32) tma_prefetch_desc(&batch.prob[g].map_d);
-            if (DSIG) tma_prefetch_desc(&batch.prob[g].map_z);
+            if (DSIG || GLU_BWD) tma_prefetch_desc(&batch.prob[g].map_z);
+            if (GLU_BWD) {
+                tma_prefetch_desc(&batch.prob[g].map_d2);
+                tma_prefetch_desc(&batch.prob[g].map_d3);
+            }
             if (EPI == EPI_GLU) {
                 tma_prefetch_desc(&batch.prob[g].map_b2);
                 tma_prefetch_desc(&batch.prob[g].map_d2);
@@ -937,29 +1000,29 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     } else {
         // ------------------------------------------------ epilogue (warps 2..9)
         const int q = warp & 3;                 // TMEM lane quarter this warp may access
-        const int half = (warp - 2) >> 2;       // which of the two warps on this quarter
+        const int half = (warp - 2) >> 2;       // which of the warps on this quarter
         // MSUB == 2: each warp of a quarter owns one 128-row sub-tile and all its
-        // chunks; MSUB == 1: the two warps take alternate chunks of the one sub-tile
+        // chunks; MSUB == 1: they take the chunks of the one sub-tile in turn
         const int sub = (MSUB == 2) ? half : 0;
         const int c_first = (MSUB == 2) ? 0 : half;
-        constexpr int C_STEP = (MSUB == 2) ? 1 : 2;
+        constexpr int C_STEP = (MSUB == 2) ? 1 : NUM_EPI_WARPS / 4;
         const int row_off = PAIR ? static_cast<int>(rank) * BM : 0;   // this CTA's rows of a pair's tile
         const int row_in_tile = row_off + sub * BM + q * 32 + lane;
-        uint8_t* ep_gen = smem_epi + (warp - 2) * EPI_WARP_BYTES;
+        uint8_t* ep_gen = smem_epi + (warp - 2) * WARP_BYTES;
         const uint32_t ep = smem_u32(ep_gen);
-        uint64_t* zbar = zfull_bar + 2 * (warp - 2);
+        uint64_t* zbar = zfull_bar + ZSLOTS * (warp - 2);
         int out_slot = 0;                       // next output box of the ring (EPI_STORE / EPI_ZH)
         int buf = 0;
         uint32_t bphase = 0;
         bool ok = true;
 
-        // 32-column chunks of unit x that hold output rows of this warp
+        // CHUNK-column chunks of unit x that hold output rows of this warp
         auto chunk_count = [&](const Unit& x) {
             const GemmParams& pu = batch.prob[x.g].p;
             if (EPI == EPI_F32 || (EPI == EPI_TAIL && x.split >= 0)) return BN / 32;   // partial tiles: all of it
             if (x.m_blk * TILE_M + row_off + sub * BM + q * 32 >= pu.M) return 0;   // this warp's 32 rows are all past the end
             const int left = pu.N - x.n_blk * BN;
-            return left >= BN ? BN / 32 : (left + 31) / 32;
+            return left >= BN ? BN / CHUNK : (left + CHUNK - 1) / CHUNK;
         };
         int cur_M = 0;                          // output rows of the tile in hand
 
@@ -1001,33 +1064,53 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             emit(map, w, col0, row0);
         };
 
-        // EPI_DSIGMA: Z boxes run one (tile, chunk) item ahead of their use
-        int zu = first_unit, zc = c_first;      // next item whose Z box is to be loaded
+        // EPI_DSIGMA: Z boxes run one (tile, chunk) item ahead of their use;
+        // EPI_GLU_BWD: so do its Y_up and Y_gate boxes (EPI_GLU_BWD_LONG: box by
+        // box, two ahead)
+        int zu = first_unit, zc = c_first;      // next item whose boxes are to be loaded
         uint32_t zphase = 0;                    // bit b: parity of the next wait on zbar[b]
-        int zload = 0, zuse = 0;
+        int zload = 0, zuse = 0;                // items loaded, items used: item i in slot i % ZSLOTS
+        int zslot_l = 0, zslot_u = 0;
+        int zsub = 0;                           // GLU_ONE: 0 = Y_up is next, 1 = Y_gate
         auto z_advance = [&]() {                // move (zu, zc) to the next item that has a chunk
             while (zu < batch.units && zc >= chunk_count(decode(batch, zu))) {
                 zu += unit_step;
                 zc = c_first;
             }
         };
-        auto z_issue = [&]() {                  // load the Z box of item (zu, zc), then step past it
+        auto z_issue = [&]() {                  // load the boxes of item (zu, zc), then step past it
             if (zu >= batch.units) return;
             const Unit x = decode(batch, zu);
-            const int b = zload & 1;
+            const int b = zslot_l;
             if (lane == 0) {
-                bulk_wait_group_read<0>();      // the stores that last read box b are done with it
-                mbar_arrive_expect_tx(&zbar[b], EPI_BOX_BYTES);
-                tma_load_2d(&batch.prob[x.g].map_z, &zbar[b], ep_gen + b * EPI_BOX_BYTES, x.n_blk * BN + zc * 32,
-                            x.m_blk * TILE_M + row_off + sub * BM + q * 32);
+                bulk_wait_group_read<0>();      // the stores that last read slot b are done with it
+                const int xc = x.n_blk * BN + zc * CHUNK, yr = x.m_blk * TILE_M + row_off + sub * BM + q * 32;
+                const GemmProblem& zp = batch.prob[x.g];
+                uint8_t* slot = ep_gen + b * epi_slot_bytes(EPI);
+                mbar_arrive_expect_tx(&zbar[b], epi_slot_bytes(EPI));
+                if (GLU_ONE) {
+                    tma_load_2d(zsub == 0 ? &zp.map_d3 : &zp.map_z, &zbar[b], slot, xc, yr);
+                } else if (GLU_BWD) {
+                    tma_load_2d(&zp.map_d3, &zbar[b], slot, xc, yr);                   // Y_up
+                    tma_load_2d(&zp.map_z, &zbar[b], slot + GLU_BOX_BYTES, xc, yr);   // Y_gate
+                } else {
+                    tma_load_2d(&zp.map_z, &zbar[b], slot, xc, yr);
+                }
             }
             ++zload;
+            if (++zslot_l == ZSLOTS) zslot_l = 0;
+            if (GLU_ONE && zsub == 0) {
+                zsub = 1;
+                return;
+            }
+            zsub = 0;
             zc += C_STEP;
             z_advance();
         };
-        if (DSIG) {
+        if (DSIG || GLU_BWD) {
             z_advance();
-            z_issue();
+#pragma unroll
+            for (int i = 0; i < ZSLOTS - 1; ++i) z_issue();
         }
 
         WorkIter it;
@@ -1153,23 +1236,89 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 }
                 continue;
             }
+            if constexpr (GLU_BWD) {
+                // dM rounded to bf16; dY_gate = bf16(dM * Y_up) in place of this
+                // row's Y_gate, dY_up = bf16(dM * Y_gate) in place of its Y_up (a
+                // bf16 product rounded once: the exact product's rounding)
+                auto free_acc = [&]() {
+                    tc_fence_before();
+                    if (PAIR)
+                        mbar_arrive_cluster(mapa_shared(smem_u32(&tempty_bar[buf]), 0));
+                    else
+                        mbar_arrive(&tempty_bar[buf]);
+                };
+#pragma unroll 1
+                for (int c = c_first; c < nch; c += C_STEP) {
+                    const int col0 = n_blk * BN + c * GLU_COLS;
+                    uint32_t v0[32], v1[32];
+                    tmem_ld_32x32b_x32(tbase + c * GLU_COLS, v0);
+                    tmem_ld_32x32b_x32(tbase + c * GLU_COLS + 32, v1);
+                    tmem_ld_wait();
+                    if (c + C_STEP >= nch) free_acc();   // the tile's last chunk is in registers
+                    uint32_t dm[32];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        dm[i] = pack_bf16x2(__uint_as_float(v0[2 * i]), __uint_as_float(v0[2 * i + 1]));
+                        dm[16 + i] = pack_bf16x2(__uint_as_float(v1[2 * i]), __uint_as_float(v1[2 * i + 1]));
+                    }
+                    const int valid = p.N - col0;
+                    const bool ragged = (p.N & 7) != 0 && valid < GLU_COLS;
+                    // this row of a box times dM, in place (or to `out`: a TMA store
+                    // would write the row padding past a ragged right edge)
+                    auto times_dm = [&](uint32_t box, __nv_bfloat16* out) {
+#pragma unroll
+                        for (int j = 0; j < GLU_COLS / 8; ++j) {
+                            const uint32_t at = box + static_cast<uint32_t>(lane * 128 + ((j ^ (lane & 7)) << 4));
+                            const uint4 y = ld_shared_v4(at);
+                            const uint4 d = make_uint4(mul_bf16x2(dm[4 * j], y.x), mul_bf16x2(dm[4 * j + 1], y.y),
+                                                       mul_bf16x2(dm[4 * j + 2], y.z), mul_bf16x2(dm[4 * j + 3], y.w));
+                            if (!ragged)
+                                st_shared_v4(at, d.x, d.y, d.z, d.w);
+                            else if (row < p.M)
+                                store_row8(out + row * p.d_ld + col0 + 8 * j, d, valid - 8 * j);
+                        }
+                    };
+                    if (!GLU_ONE) z_issue();   // the next chunk's boxes, into the slot stored from a chunk ago
+#pragma unroll 1
+                    for (int f = 0; f < (GLU_ONE ? 2 : 1); ++f) {
+                        const int b = zslot_u;
+                        ok = wait_bounded(&zbar[b], (zphase >> b) & 1u, wc, ST_TIMEOUT_EPILOGUE);
+                        zphase ^= 1u << b;
+                        ++zuse;
+                        if (++zslot_u == ZSLOTS) zslot_u = 0;
+                        if (!ok) break;
+                        const uint32_t box = ep + b * epi_slot_bytes(EPI);
+                        times_dm(box, f == 0 ? p.d_ptr : p.d2_ptr);
+                        if (!GLU_ONE) times_dm(box + GLU_BOX_BYTES, p.d2_ptr);
+                        if (GLU_ONE) {
+                            z_issue();   // two boxes ahead, into the slot stored from a box ago
+                            // the caller may hand Y_gate's storage to dY_gate: its box
+                            // has landed before dY_gate is stored
+                            if (f == 0) ok = wait_bounded(&zbar[zslot_u], (zphase >> zslot_u) & 1u, wc, ST_TIMEOUT_EPILOGUE);
+                            if (!ok) break;
+                        }
+                        fence_proxy_async_smem();   // the slot's writes (ragged: reads) before its stores (next load)
+                        __syncwarp();
+                        if (!ragged && lane == 0) {
+                            tma_store_2d(f == 0 ? map_d : map_d2, box, col0, row0);
+                            if (!GLU_ONE) tma_store_2d(map_d2, box + GLU_BOX_BYTES, col0, row0);
+                            bulk_commit_group();
+                        }
+                    }
+                    if (!ok) break;
+                }
+                if (!ok) break;
+                if (nch <= c_first) free_acc();   // no chunk of this tile is this warp's
+                if (++buf == 2) {
+                    buf = 0;
+                    bphase ^= 1u;
+                }
+                continue;
+            }
 #pragma unroll 1
             for (int c = c_first; c < nch; c += C_STEP) {
                 const int col0 = n_blk * BN + c * 32;
                 if (DSIG) z_issue();   // the next item's Z box, while this one is processed
-                // EPI_GLU_BWD: this row's Y_gate and Y_up chunk, loaded ahead of the accumulator
-                uint4 yg[4], yu[4];
-                if constexpr (EPI == EPI_GLU_BWD) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        yg[j] = yu[j] = make_uint4(0u, 0u, 0u, 0u);
-                        if (row < p.M && col0 + 8 * j < p.N) {   // 8-column vectors inside the padded row
-                            const long long off = static_cast<long long>(row) * p.d_ld + col0 + 8 * j;
-                            yg[j] = __ldg(reinterpret_cast<const uint4*>(p.yg_ptr + off));
-                            yu[j] = __ldg(reinterpret_cast<const uint4*>(p.yu_ptr + off));
-                        }
-                    }
-                }
                 uint32_t v[32];
                 uint32_t v2[32];   // EPI_GLU: the same chunk of the up accumulator
                 tmem_ld_32x32b_x32(tbase + c * 32, v);
@@ -1215,30 +1364,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         put(p, map_d2, p.d2_ptr, wg, col0, row0, row);
                         put(p, &batch.prob[x.g].map_d3, p.d3_ptr, wu, col0, row0, row);
                     }
-                } else if (EPI == EPI_GLU_BWD) {
-                    // dM rounded to bf16; dY_gate = bf16(dM * Y_up), dY_up = bf16(dM * Y_gate)
-                    uint32_t dm[16], gw[16], uw[16];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        gw[4 * j] = yg[j].x;
-                        gw[4 * j + 1] = yg[j].y;
-                        gw[4 * j + 2] = yg[j].z;
-                        gw[4 * j + 3] = yg[j].w;
-                        uw[4 * j] = yu[j].x;
-                        uw[4 * j + 1] = yu[j].y;
-                        uw[4 * j + 2] = yu[j].z;
-                        uw[4 * j + 3] = yu[j].w;
-                    }
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        dm[j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
-                        w[j] = pack_bf16x2(bf16_lo(dm[j]) * bf16_lo(uw[j]), bf16_hi(dm[j]) * bf16_hi(uw[j]));
-                    }
-                    put(p, map_d, p.d_ptr, w, col0, row0, row);      // dY_gate
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        w[j] = pack_bf16x2(bf16_lo(dm[j]) * bf16_lo(gw[j]), bf16_hi(dm[j]) * bf16_hi(gw[j]));
-                    put(p, map_d2, p.d2_ptr, w, col0, row0, row);    // dY_up
                 } else if (EPI == EPI_ZH) {
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
@@ -1261,10 +1386,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         emit(p.h_only ? map_d : map_d2, w, col0, row0);
                     }
                 } else if (DSIG) {
-                    const int b = zuse & 1;
+                    const int b = zslot_u;
                     const bool zok = wait_bounded(&zbar[b], (zphase >> b) & 1u, wc, ST_TIMEOUT_EPILOGUE);
                     zphase ^= 1u << b;
                     ++zuse;
+                    if (++zslot_u == ZSLOTS) zslot_u = 0;
                     if (!zok) {
                         ok = false;
                         break;
@@ -1339,7 +1465,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         }
         // Z boxes still in flight (issued ahead, or for items the loop left early)
         while (zuse < zload) {
-            const int b = zuse & 1;
+            const int b = zslot_u;
             const uint64_t t0 = global_timer_ns();
             while (!mbar_try_wait(&zbar[b], (zphase >> b) & 1u)) {
                 if (global_timer_ns() - t0 > WAIT_LIMIT_NS) {
@@ -1349,6 +1475,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             }
             zphase ^= 1u << b;
             ++zuse;
+            if (++zslot_u == ZSLOTS) zslot_u = 0;
         }
         if (lane == 0) bulk_wait_group_all();   // every output store has landed
     }

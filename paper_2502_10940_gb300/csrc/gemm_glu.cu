@@ -14,7 +14,6 @@ template cudaError_t launch_gemm<128, 1, false, false, EPI_GLU>(const GemmBatch&
 template cudaError_t launch_gemm<256, 1, false, false, EPI_GLU, true>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<128, 1, false, false, EPI_GLU, true>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<128, 1, false, true, EPI_GLU_BWD>(const GemmBatch&, int, bool, cudaStream_t);
-template cudaError_t launch_gemm<256, 1, false, true, EPI_GLU_BWD>(const GemmBatch&, int, bool, cudaStream_t);
-template cudaError_t launch_gemm<128, 2, false, true, EPI_GLU_BWD>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<256, 1, false, true, EPI_GLU_BWD, true>(const GemmBatch&, int, bool, cudaStream_t);
+template cudaError_t launch_gemm<256, 1, false, true, EPI_GLU_BWD_LONG, true>(const GemmBatch&, int, bool, cudaStream_t);
 }  // namespace cola

@@ -77,7 +77,7 @@ cudaError_t launch_sigma(const void* Z, void* H, long long elems, int sigma, int
 template <int BN, int MSUB, bool A_MN, bool B_MN, int EPI, bool PAIR, int SIG>
 cudaError_t launch_gemm(const GemmBatch& batch, int grid, bool pdl, cudaStream_t stream)
 {
-    constexpr int smem = GemmCfg<BN, MSUB, PAIR>::SMEM_BYTES;
+    constexpr int smem = EpiGemmCfg<BN, MSUB, PAIR, EPI>::SMEM_BYTES;
     auto kern = gemm_kernel<BN, MSUB, A_MN, B_MN, EPI, PAIR, SIG>;
     // the opt-in shared-memory size is a per-device function attribute; host
     // threads may launch concurrently, so the set of configured devices is atomic

@@ -60,6 +60,13 @@ bool map_box32(CUtensorMap* m, const void* base, int64_t cols, int64_t rows, int
     return make_map(m, base, cols, rows, ld, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
+// Box of 32 rows x 64 columns (128-byte rows, 128-byte swizzle): the chunks of
+// the gated dX epilogue.
+bool map_box64(CUtensorMap* m, const void* base, int64_t cols, int64_t rows, int64_t ld)
+{
+    return make_map(m, base, cols, rows, ld, GLU_COLS, 32, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
 // K-major operand: rows are the M (or N) index, k contiguous: box {64, rows_per_tile}.
 // MN-major operand: rows are k, the M (or N) index contiguous: box {64, 64}.
 bool map_kmajor(CUtensorMap* m, const void* base, int64_t k_extent, int64_t mn_extent, int64_t ld, int tile_rows)
@@ -383,21 +390,29 @@ cudaError_t dispatch_sig(int bn, int msub, GemmBatch& b, int sms, cudaStream_t s
     b.units = units;
     const bool pdl = flops < 64e9;
     // the split-K forward GEMMs of small launches (K-major fp32 partials) run
-    // on single-CTA 128-row tiles only
+    // on single-CTA 128-row tiles only; the gated dX GEMM on CTA pairs or on
+    // 128 x 128 tiles (its long-K form on pairs only)
     constexpr bool small_only = EPI == EPI_F32 && !A_MN;
+    constexpr bool glu_bwd = epi_glu_bwd(EPI);
     if constexpr (!small_only) {
         if (msub == TILE_PAIR && bn == 256) {
             const int pairs = units < sms / 2 ? units : sms / 2;
             return launch_gemm<256, 1, A_MN, B_MN, EPI, true, SIG>(b, 2 * pairs, pdl, s);
         }
     }
-    if (msub != 1 && (bn == 256 || small_only)) return cudaErrorInvalidValue;   // planned tiles exist as above only
+    // planned tiles exist as above and below only
+    if (msub != 1 && (bn == 256 || small_only || glu_bwd)) return cudaErrorInvalidValue;
     const int grid = units < sms ? units : sms;
-    if (bn == 256) return launch_gemm<256, 1, A_MN, B_MN, EPI, false, SIG>(b, grid, pdl, s);
-    if constexpr (!small_only) {
+    if constexpr (glu_bwd) {
+        if (bn == 256) return cudaErrorInvalidValue;
+    } else {
+        if (bn == 256) return launch_gemm<256, 1, A_MN, B_MN, EPI, false, SIG>(b, grid, pdl, s);
+    }
+    if constexpr (!small_only && !glu_bwd) {
         if (msub != 1) return launch_gemm<128, 2, A_MN, B_MN, EPI, false, SIG>(b, grid, pdl, s);
     }
-    return launch_gemm<128, 1, A_MN, B_MN, EPI, false, SIG>(b, grid, pdl, s);
+    if constexpr (EPI == EPI_GLU_BWD_LONG) return cudaErrorInvalidValue;
+    else return launch_gemm<128, 1, A_MN, B_MN, EPI, false, SIG>(b, grid, pdl, s);
 }
 
 // The launch of a batch whose epilogue applies sigma (EPI_ZH, EPI_DSIGMA,
