@@ -171,7 +171,17 @@ constexpr int epi_slot_bytes(int epi)
 {
     return epi == EPI_GLU_BWD ? 2 * GLU_BOX_BYTES : epi == EPI_GLU_BWD_LONG ? GLU_BOX_BYTES : EPI_BOX_BYTES;
 }
-constexpr int epi_warp_bytes(int epi) { return epi_glu_bwd(epi) ? epi_slots(epi) * epi_slot_bytes(epi) : EPI_WARP_BYTES; }
+// EPI_GLU: one 64-column output box per warp, staged again only when its store
+// has read it, which leaves room for six operand stages.  Training at r = 512,
+// 65536 x 5461: 875 us with 256 x 128 pair tiles and 32-column boxes, 699 us
+// with 256 x 256 tiles whose halves are handed over apart and this box (four
+// stages: 733 us); 65536 x 2736 (r = 256, single CTAs) 274 -> 250 us with one
+// box, 322 us with three.
+constexpr int epi_warp_bytes(int epi)
+{
+    return epi_glu_bwd(epi) ? epi_slots(epi) * epi_slot_bytes(epi)
+                            : (epi == EPI_GLU ? GLU_BOX_BYTES : EPI_WARP_BYTES);
+}
 
 // A CTA tile is MSUB x 128 rows by BN columns: MSUB = 2 runs two M = 128
 // MMAs per k-step that share one B tile (halving the B-operand traffic per
@@ -196,7 +206,7 @@ struct GemmCfg {
     static constexpr int BAR_BYTES = 512;        // <= 47 mbarriers, the TMEM address, the abort flag, a count
     static constexpr int SMEM_LIMIT = 232448;   // opt-in maximum per CTA
     static constexpr int STAGES_FIT = (SMEM_LIMIT - 1024 - BAR_BYTES - EPI_BYTES) / STAGE_BYTES;
-    static constexpr int STAGES = STAGES_FIT > 8 ? 8 : STAGES_FIT;
+        static constexpr int STAGES = STAGES_FIT > 8 ? 8 : STAGES_FIT;
     static constexpr int TMEM_COLS = (BUFS * ACC_COLS <= 128) ? 128 : (BUFS * ACC_COLS <= 256 ? 256 : 512);
     static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + EPI_BYTES + BAR_BYTES;
     static_assert(SMEM_BYTES <= SMEM_LIMIT, "shared memory budget");
@@ -608,6 +618,16 @@ __device__ __forceinline__ void stage_row(uint32_t box, int lane, const uint32_t
     for (int j = 0; j < 4; ++j) st_shared_v4(box + box64_off(lane, j), w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
 }
 
+// The same for a box of 32 rows x 64 columns with the 128-byte swizzle; w(j)
+// is the row's j-th packed pair.
+template <class W>
+__device__ __forceinline__ void stage_row128(uint32_t box, int lane, W&& w)
+{
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        st_shared_v4(box + lane * 128 + ((j ^ (lane & 7)) << 4), w(4 * j), w(4 * j + 1), w(4 * j + 2), w(4 * j + 3));
+}
+
 // Store the first `valid` (up to 8) of 8 packed bf16 at d (16-byte aligned).
 __device__ __forceinline__ void store_row8(__nv_bfloat16* d, const uint4& w, int valid)
 {
@@ -628,11 +648,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     gemm_kernel(const __grid_constant__ GemmBatch batch)
 {
     // EPI_GLU with 256-column tiles: the gate and up accumulators of one tile
-    // fill TMEM, so there is one tile slot, and its two accumulators are
-    // released apart: the epilogue copies the gate half to registers and frees
-    // it at once (tempty_bar[0]), so the MMAs of the next tile's gate half
-    // overlap this tile's up-half epilogue; the up half is freed when stored
-    // (tempty_bar[1]).
+    // fill TMEM, so there is one tile slot, and its two halves are handed over
+    // apart (tfull / tempty 0: gate, 1: up): the epilogue copies the gate half
+    // to registers while the up half's MMAs run, so the next tile's MMAs follow
+    // without a gap
     constexpr bool GLU_SPLIT = EPI == EPI_GLU && BN == 256;
     // EPI_STORE on a CTA pair: the accumulator is freed as soon as the
     // epilogue holds the tile's values in registers, before its stores
@@ -651,7 +670,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     constexpr bool GLU_ONE = EPI == EPI_GLU_BWD_LONG;   // one box per slot
     constexpr int WARP_BYTES = epi_warp_bytes(EPI);
     constexpr int ZSLOTS = epi_slots(EPI);          // side-input slots per epilogue warp
-    constexpr int CHUNK = GLU_BWD ? GLU_COLS : 32;      // columns of one epilogue chunk
+    constexpr int CHUNK = GLU_BWD || EPI == EPI_GLU ? GLU_COLS : 32;   // columns of one epilogue chunk
     constexpr int STAGES = C::STAGES;
     constexpr int TILE_M = C::TILE_M;
     extern __shared__ uint8_t smem_raw[];
@@ -965,6 +984,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         umma_commit_pair(&empty_bar[stage], 0x3);
                     else
                         umma_commit(&empty_bar[stage]);
+                    if (GLU_SPLIT && kb == half - 1) {   // the gate accumulator is ready
+                        if (PAIR)
+                            umma_commit_pair(&tfull_bar[0], 0x3);
+                        else
+                            umma_commit(&tfull_bar[0]);
+                    }
                     if (++stage == STAGES) {
                         stage = 0;
                         phase ^= 1u;
@@ -973,9 +998,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 if (!ok) break;
                 // accumulator ready for the epilogue (of both CTAs of a pair)
                 if (PAIR)
-                    umma_commit_pair(&tfull_bar[buf], 0x3);
+                    umma_commit_pair(&tfull_bar[GLU_SPLIT ? 1 : buf], 0x3);
                 else
-                    umma_commit(&tfull_bar[buf]);
+                    umma_commit(&tfull_bar[GLU_SPLIT ? 1 : buf]);
                 if (GLU_SPLIT) {
                     bphase ^= 1u;   // one slot: buf stays 0
                 } else if (++buf == 2) {
@@ -1129,54 +1154,94 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             tc_fence_after();
             const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
                                    static_cast<uint32_t>((GLU_SPLIT ? 0 : buf * C::ACC_COLS) + sub * BN);
-            if constexpr (GLU_SPLIT) {
-                // the gate half of this warp's chunks into registers, then free it
-                uint32_t gsave[BN / 64][16];
+            if constexpr (EPI == EPI_GLU) {
+                // the gate half of this warp's chunks into registers as bf16, its
+                // accumulator freed at once; then, chunk by chunk, the up half and
+                // the stores.  The up accumulator is freed with its last chunk read,
+                // which is before the next tile's MMAs come to it
+                constexpr int NC = BN / (C_STEP * GLU_COLS);
+                uint32_t g[NC][32];
+                auto take = [&](uint32_t taddr, uint32_t (&w)[32]) {
 #pragma unroll
-                for (int i = 0; i < BN / 64; ++i) {
-                    const int c = c_first + C_STEP * i;
-                    if (c < nch) {
+                    for (int h = 0; h < 2; ++h) {
                         uint32_t v[32];
-                        tmem_ld_32x32b_x32(tbase + c * 32, v);
+                        tmem_ld_32x32b_x32(taddr + 32 * h, v);
                         tmem_ld_wait();
 #pragma unroll
                         for (int j = 0; j < 16; ++j)
-                            gsave[i][j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+                            w[16 * h + j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
                     }
-                }
-                tc_fence_before();
-                if (PAIR)
-                    mbar_arrive_cluster(mapa_shared(smem_u32(&tempty_bar[0]), 0));
-                else
-                    mbar_arrive(&tempty_bar[0]);
-                // the up half: M = bf16(Y_gate * Y_up), and Y_gate, Y_up when training
+                };
+                auto free_acc = [&](uint64_t* bar) {
+                    tc_fence_before();
+                    if (PAIR)
+                        mbar_arrive_cluster(mapa_shared(smem_u32(bar), 0));
+                    else
+                        mbar_arrive(bar);
+                };
 #pragma unroll
-                for (int i = 0; i < BN / 64; ++i) {
+                for (int i = 0; i < NC; ++i)
+                    if (c_first + C_STEP * i < nch) take(tbase + (c_first + C_STEP * i) * GLU_COLS, g[i]);
+                if (GLU_SPLIT) {
+                    free_acc(&tempty_bar[0]);
+                    if (!wait_bounded(&tfull_bar[1], bphase, wc, ST_TIMEOUT_EPILOGUE)) break;
+                    tc_fence_after();
+                }
+                uint64_t* const up_free = &tempty_bar[GLU_SPLIT ? 1 : buf];
+                if (c_first >= nch) free_acc(up_free);   // no chunk of this tile is this warp's
+#pragma unroll
+                for (int i = 0; i < NC; ++i) {
                     const int c = c_first + C_STEP * i;
                     if (c < nch) {
-                        const int col0 = n_blk * BN + c * 32;
-                        uint32_t v[32];
-                        tmem_ld_32x32b_x32(tbase + BN + c * 32, v);
-                        tmem_ld_wait();
-                        uint32_t wu[16], w[16];
+                        uint32_t u[32];
+                        take(tbase + BN + c * GLU_COLS, u);
+                        if (c + C_STEP >= nch) free_acc(up_free);
+                        // M = bf16(Y_gate * Y_up) of the rounded outputs (a bf16 product
+                        // rounded once: the exact product's rounding); Y_gate and Y_up
+                        // too when training
+                        const int col0 = n_blk * BN + c * GLU_COLS;
+                        const int valid = p.N - col0;
+                        auto m = [&](int j) { return mul_bf16x2(g[i][j], u[j]); };
+                        auto yg = [&](int j) { return g[i][j]; };
+                        auto yu = [&](int j) { return u[j]; };
+                        if ((p.N & 7) != 0 && valid < GLU_COLS) {
+                            // a TMA store would write the row padding past a ragged right edge
+                            if (row < p.M) {
+                                const long long off = row * p.d_ld + col0;
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            wu[j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
-                            w[j] = pack_bf16x2(bf16_lo(gsave[i][j]) * bf16_lo(wu[j]), bf16_hi(gsave[i][j]) * bf16_hi(wu[j]));
-                        }
-                        put(p, map_d, p.d_ptr, w, col0, row0, row);
-                        if (p.has_d2) {
-                            put(p, map_d2, p.d2_ptr, gsave[i], col0, row0, row);
-                            put(p, &batch.prob[x.g].map_d3, p.d3_ptr, wu, col0, row0, row);
+                                for (int j = 0; j < GLU_COLS / 8; ++j) {
+                                    auto at = [&](auto&& w) {
+                                        return make_uint4(w(4 * j), w(4 * j + 1), w(4 * j + 2), w(4 * j + 3));
+                                    };
+                                    store_row8(p.d_ptr + off + 8 * j, at(m), valid - 8 * j);
+                                    if (p.has_d2) {
+                                        store_row8(p.d2_ptr + off + 8 * j, at(yg), valid - 8 * j);
+                                        store_row8(p.d3_ptr + off + 8 * j, at(yu), valid - 8 * j);
+                                    }
+                                }
+                            }
+                        } else {
+                            auto emit64 = [&](const CUtensorMap* map, auto&& w) {
+                                if (lane == 0) bulk_wait_group_read<0>();   // the box's previous store has read it
+                                __syncwarp();
+                                stage_row128(ep, lane, w);
+                                fence_proxy_async_smem();
+                                store_box(map, ep, col0, row0);
+                            };
+                            emit64(map_d, m);
+                            if (p.has_d2) {
+                                emit64(map_d2, yg);
+                                emit64(&batch.prob[x.g].map_d3, yu);
+                            }
                         }
                     }
                 }
-                tc_fence_before();
-                if (PAIR)
-                    mbar_arrive_cluster(mapa_shared(smem_u32(&tempty_bar[1]), 0));
-                else
-                    mbar_arrive(&tempty_bar[1]);
-                bphase ^= 1u;
+                if (GLU_SPLIT) {
+                    bphase ^= 1u;   // one slot: buf stays 0
+                } else if (++buf == 2) {
+                    buf = 0;
+                    bphase ^= 1u;
+                }
                 continue;
             }
             if constexpr (EARLY_FREE) {
@@ -1320,9 +1385,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 const int col0 = n_blk * BN + c * 32;
                 if (DSIG) z_issue();   // the next item's Z box, while this one is processed
                 uint32_t v[32];
-                uint32_t v2[32];   // EPI_GLU: the same chunk of the up accumulator
                 tmem_ld_32x32b_x32(tbase + c * 32, v);
-                if constexpr (EPI == EPI_GLU) tmem_ld_32x32b_x32(tbase + BN + c * 32, v2);
                 tmem_ld_wait();
                 if (EPI == EPI_F32 || (EPI == EPI_TAIL && split >= 0)) {
                     float* dst = nullptr;
@@ -1349,21 +1412,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     for (int j = 0; j < 16; ++j)
                         w[j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
                     put(p, map_d, p.d_ptr, w, col0, row0, row);
-                } else if (EPI == EPI_GLU) {
-                    // Y_gate, Y_up rounded to bf16; M = bf16(Y_gate * Y_up) of the rounded
-                    // values (their product is exact in fp32)
-                    uint32_t wg[16], wu[16];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        wg[j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
-                        wu[j] = pack_bf16x2(__uint_as_float(v2[2 * j]), __uint_as_float(v2[2 * j + 1]));
-                        w[j] = pack_bf16x2(bf16_lo(wg[j]) * bf16_lo(wu[j]), bf16_hi(wg[j]) * bf16_hi(wu[j]));
-                    }
-                    put(p, map_d, p.d_ptr, w, col0, row0, row);
-                    if (p.has_d2) {                 // training: Y_gate and Y_up for the backward
-                        put(p, map_d2, p.d2_ptr, wg, col0, row0, row);
-                        put(p, &batch.prob[x.g].map_d3, p.d3_ptr, wu, col0, row0, row);
-                    }
                 } else if (EPI == EPI_ZH) {
 #pragma unroll
                     for (int j = 0; j < 16; ++j)
