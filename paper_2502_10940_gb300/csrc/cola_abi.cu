@@ -299,6 +299,7 @@ cola_status_t run_batch(int kind, int bn, int msub, const GemmProblem* probs, co
 }  // namespace
 
 cudaError_t launch_splitk_cluster(const CredBatch& b, bool pdl, cudaStream_t stream);
+cudaError_t launch_thin(const ThinBatch& b, int kind, int sigma, cudaStream_t stream);
 
 namespace {
 
@@ -463,15 +464,119 @@ std::atomic<int> g_fused_bwd{1};
 // 128-row tile per SM, and not split over K (small launches keep the
 // split-K forward).  Measured at 2048 tokens: -10 to -13 % against the two
 // GEMMs; at 65536 tokens it was 5-13 % slower, so larger launches keep them.
-bool fused_fwd_applies(const Shape& s, int sms)
+bool fused_fwd_form(const Shape& s, int sms)
 {
-    if (!g_fused_fwd.load(std::memory_order_relaxed) || (s.r != 64 && s.r != 128)) return false;
+    if (s.r != 64 && s.r != 128) return false;
     if ((s.n + BM - 1) / BM > sms) return false;
     if (heavy_gemm(s.n, s.r, s.d_in) || heavy_gemm(s.n, s.d_out, s.r)) return false;
     GemmParams p1 = base_params(s.n, s.r, s.d_in, choose_bn_for(s.n, s.r, s.d_in), 1);
     if (small_launch_splits(p1.m_tiles * p1.n_tiles, p1.k_blocks, sms) > 1) return false;
     GemmParams p2 = base_params(s.n, s.d_out, s.r, choose_bn_for(s.n, s.d_out, s.r), 1);
     return small_launch_splits(p2.m_tiles * p2.n_tiles, p2.k_blocks, sms) == 1;
+}
+
+bool fused_fwd_applies(const Shape& s, int sms)
+{
+    return g_fused_fwd.load(std::memory_order_relaxed) && fused_fwd_form(s, sms);
+}
+
+// The forward GEMMs of a few tokens run on the thin kernels (thin.cuh), except
+// the lone layers that have the single-kernel form, whose two GEMMs have to
+// match it bit for bit.  Above 32 tokens their epilogue (a token a warp at a
+// time) needs the splits that r >= 256 allows: blocks of 64 tokens, r = 256
+// 46.5 -> 45.1 us, but a gated MLP of 57 tokens, r = 128 23.7 -> 25.3 us.
+bool thin_applies(const Shape& s, int count, int sms)
+{
+    if (s.n > THIN_MAX_TOKENS || (s.n > 32 && s.r < 256)) return false;
+    return !(count == 1 && fused_fwd_form(s, sms));
+}
+
+// F1 of a few tokens: Z = X A^T (stored when not null), H = sigma(Z), N = r or
+// count r features
+cola_status_t run_thin_f1(const Shape& s, int sigma, int64_t N, const void* X, const void* A, void* Z, void* H,
+                          unsigned int* status, int sms, cudaStream_t st)
+{
+    ThinBatch b;
+    std::memset(&b, 0, sizeof b);
+    b.count = 1;
+    b.n = static_cast<int>(s.n);
+    b.tiles = static_cast<int>((N + BM - 1) / BM);
+    b.k_blocks = static_cast<int>((s.d_in + BK - 1) / BK);
+    thin_splits(b, false, sms);
+    COLA_MAP(map_kmajor(&b.map_t, X, s.d_in, s.n, s.ld_x, b.NT));
+    ThinProblem& P = b.prob[0];
+    COLA_MAP(map_kmajor(&P.map_w, A, s.d_in, N, s.ld_a, BM));
+    P.M = static_cast<int>(N);
+    P.o0 = static_cast<__nv_bfloat16*>(Z);
+    P.o1 = static_cast<__nv_bfloat16*>(H);
+    P.ldo = N;
+    b.status = status;
+    const int64_t mnk[1][3] = {{s.n, N, s.d_in}};
+    return launched(traced(COLA_KERNEL_FWD_ZH, 1, mnk, b.S, (Z ? 1 : 0) | TRACE_CLUSTER, st,
+                           [&] { return launch_thin(b, THIN_ZH, sigma, st); }));
+}
+
+// F2 of a few tokens: Y_j = H_j B_j^T for `count` projections, H_j the column
+// blocks of H (pitch ldh).  Follows another kernel of the same call, so its
+// weights may be loaded ahead of the wait for it.
+cola_status_t run_thin_f2(const Shape& s, int count, const void* H, int64_t ldh, const void* const* B, void* const* Y,
+                          unsigned int* status, int sms, cudaStream_t st)
+{
+    ThinBatch b;
+    std::memset(&b, 0, sizeof b);
+    b.count = count;
+    b.n = static_cast<int>(s.n);
+    const int per = static_cast<int>((s.d_out + BM - 1) / BM);
+    b.tiles = count * per;
+    b.k_blocks = static_cast<int>(s.r / BK);
+    thin_splits(b, false, sms);
+    COLA_MAP(map_kmajor(&b.map_t, H, ldh, s.n, ldh, b.NT));
+    int64_t mnk[THIN_MAX_PROBS][3];
+    for (int j = 0; j < count; ++j) {
+        ThinProblem& P = b.prob[j];
+        COLA_MAP(map_kmajor(&P.map_w, B[j], s.r, s.d_out, s.r, BM));
+        P.M = static_cast<int>(s.d_out);
+        P.tile_begin = j * per;
+        P.t_x = static_cast<int>(j * s.r);
+        P.o0 = static_cast<__nv_bfloat16*>(Y[j]);
+        P.ldo = s.ld_y;
+        mnk[j][0] = s.n;
+        mnk[j][1] = s.d_out;
+        mnk[j][2] = s.r;
+    }
+    b.early_weights = 1;
+    b.status = status;
+    return launched(traced(COLA_KERNEL_FWD_Y, count, mnk, b.S, TRACE_CLUSTER, st,
+                           [&] { return launch_thin(b, THIN_STORE, SIG_IDENTITY, st); }));
+}
+
+// The gated product of a few tokens: M = (H_gate B_gate^T) * (H_up B_up^T)
+cola_status_t run_thin_glu(const Shape& s, const void* H_cat, const void* Bg, const void* Bu, void* M, void* Yg, void* Yu,
+                           unsigned int* status, int sms, cudaStream_t st)
+{
+    ThinBatch b;
+    std::memset(&b, 0, sizeof b);
+    b.count = 1;
+    b.n = static_cast<int>(s.n);
+    b.tiles = static_cast<int>((s.d_out + BM - 1) / BM);
+    b.k_blocks = static_cast<int>(s.r / BK);
+    thin_splits(b, true, sms);
+    const int64_t K2 = 2 * s.r;
+    COLA_MAP(map_kmajor(&b.map_t, H_cat, K2, s.n, K2, b.NT));
+    ThinProblem& P = b.prob[0];
+    COLA_MAP(map_kmajor(&P.map_w, Bg, s.r, s.d_out, s.r, BM));
+    COLA_MAP(map_kmajor(&P.map_w2, Bu, s.r, s.d_out, s.r, BM));
+    P.M = static_cast<int>(s.d_out);
+    P.t_x2 = static_cast<int>(s.r);
+    P.o0 = static_cast<__nv_bfloat16*>(M);
+    P.o1 = static_cast<__nv_bfloat16*>(Yg);
+    P.o2 = static_cast<__nv_bfloat16*>(Yu);
+    P.ldo = s.ld_y;
+    b.early_weights = 1;
+    b.status = status;
+    const int64_t mnk[1][3] = {{s.n, s.d_out, K2}};
+    return launched(traced(COLA_KERNEL_FWD_GLU, 1, mnk, b.S, (Yg ? 1 : 0) | TRACE_CLUSTER, st,
+                           [&] { return launch_thin(b, THIN_GLU, SIG_IDENTITY, st); }));
 }
 
 // The single-kernel dZ + dX applies on the same terms: r = 64 or 128, at
@@ -936,10 +1041,14 @@ cola_status_t cola_fwd(const cola_desc_t* desc, const void* X, const void* A, co
     const size_t part_bytes = L.total - L.part_off;
     if (fused_fwd_applies(s, sms))
         return run_fused_fwd(s, desc->sigma, X, A, B, Y, Z_save, H_save, status, sms, st);
-    COLA_TRY(run_f1(s, desc->sigma, s.r, X, A, Z_save, H, s.r, part, part_bytes, status, sms, st));
     const void* Hs[1] = {H};
     const void* Bs[1] = {B};
     void* Ys[1] = {Y};
+    if (thin_applies(s, 1, sms)) {
+        COLA_TRY(run_thin_f1(s, desc->sigma, s.r, X, A, Z_save, H, status, sms, st));
+        return run_thin_f2(s, 1, H, s.r, Bs, Ys, status, sms, st);
+    }
+    COLA_TRY(run_f1(s, desc->sigma, s.r, X, A, Z_save, H, s.r, part, part_bytes, status, sms, st));
     return run_f2(s, 1, Hs, s.r, Bs, Ys, part, part_bytes, status, sms, st);
 }
 
@@ -1043,6 +1152,10 @@ cola_status_t cola_fwd_gate_up(const cola_desc_t* desc, const void* X, const voi
     uint8_t* H = desc->mode != COLA_MODE_COLA ? wsb(ws) + L.h_off : static_cast<uint8_t*>(H_cat);
     float* part = reinterpret_cast<float*>(wsb(ws) + L.part_off);
     const size_t part_bytes = L.total - L.part_off;
+    if (thin_applies(s, 2, sms)) {
+        COLA_TRY(run_thin_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, status, sms, st));
+        return run_thin_glu(s, H, B_gate, B_up, M, Y_gate, Y_up, status, sms, st);
+    }
     COLA_TRY(run_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, R, part, part_bytes, status, sms, st));
     return run_glu(s, H, R, B_gate, B_up, M, Y_gate, Y_up, status, sms, st);
 }
@@ -1068,6 +1181,10 @@ cola_status_t cola_fwd_shared_x(const cola_desc_t* desc, int32_t count, const vo
     uint8_t* H = desc->mode != COLA_MODE_COLA ? wsb(ws) + L.h_off : static_cast<uint8_t*>(H_cat);
     float* part = reinterpret_cast<float*>(wsb(ws) + L.part_off);
     const size_t part_bytes = L.total - L.part_off;
+    if (thin_applies(s, count, sms)) {
+        COLA_TRY(run_thin_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, status, sms, st));
+        return run_thin_f2(s, count, H, R, B, Y, status, sms, st);
+    }
     COLA_TRY(run_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, R, part, part_bytes, status, sms, st));
     const void* Hs[3] = {H, H + slice, H + 2 * slice};
     return run_f2(s, count, Hs, R, B, Y, part, part_bytes, status, sms, st);
@@ -1157,6 +1274,7 @@ cola_status_t cola_recompute_up(const cola_desc_t* desc, int32_t count, const vo
     COLA_TRY(launched(traced(COLA_KERNEL_SIGMA, 1, mnk, 1, 0, st, [&] {
         return launch_sigma(Z_cat, H, static_cast<long long>(s.n) * R, desc->sigma, sms, st);
     })));
+    if (thin_applies(s, count, sms)) return run_thin_f2(s, count, H, R, B, Y, status, sms, st);
     const size_t slice = static_cast<size_t>(s.r) * 2;
     const void* Hs[3] = {H, H + slice, H + 2 * slice};
     float* part = reinterpret_cast<float*>(wsb(ws) + L.part_off);

@@ -11,6 +11,7 @@
 
 #include "gemm_launch.cuh"
 #include "splitk_cluster.cuh"
+#include "thin.cuh"
 
 namespace cola {
 namespace {
@@ -216,6 +217,31 @@ int cluster_splits(int tiles, int k_blocks, int sms)
     if (s > MAX_CLUSTER) s = MAX_CLUSTER;
     if (s > k_blocks / 4) s = k_blocks / 4;
     return s < 1 ? 1 : s;
+}
+
+// Split of a thin launch (thin.cuh): `tiles` 128-row weight tiles over k_blocks
+// (per half of a gated product).  Clusters of up to 16 CTAs with at least two
+// k-blocks each, 1.6 CTAs per SM at most (measured, 7B-shaped block of one
+// token: 61.3 us at 1.25, 58.6 at 1.6, 64.4 at 2; 1B-shaped, 32 tokens: 45.1,
+// 44.0, 44.9); the operand ring as deep as lets two CTAs, or one and a CTA of
+// the kernel before, share an SM.
+void thin_splits(ThinBatch& b, bool glu, int sms)
+{
+    b.NT = (b.n + 15) / 16 * 16;
+    int s = sms * 8 / 5 / b.tiles;
+    if (s > (b.k_blocks + 1) / 2) s = (b.k_blocks + 1) / 2;
+    if (s > THIN_MAX_CLUSTER) s = THIN_MAX_CLUSTER;
+    if (s < 1) s = 1;
+    b.kps = (b.k_blocks + s - 1) / s;
+    b.S = (b.k_blocks + b.kps - 1) / b.kps;   // no empty split
+    b.TB = (b.n + b.S - 1) / b.S;
+    constexpr int budget = 110 * 1024;
+    const int left = budget - 1024 - THIN_BAR_BYTES - thin_recv_bytes(b.S, b.TB, glu);
+    b.stages = left / thin_stage_bytes(b.NT);
+    const int iters = b.kps * (glu ? 2 : 1);
+    if (b.stages > iters) b.stages = iters;
+    if (b.stages > THIN_MAX_STAGES) b.stages = THIN_MAX_STAGES;
+    if (b.stages < 2) b.stages = 2;
 }
 
 int64_t partial_elems(const GemmParams& p, int bn, int msub)
