@@ -163,7 +163,7 @@ int64_t fwd_part_elems(const cola_desc_t& d, int nproj, int sms)
 {
     int64_t need = 0;
     const int64_t R = nproj * d.r;
-    const int bn1 = choose_bn_for(d.n, R, d.d_in);
+    const int bn1 = fill_bn(d.n, R, d.d_in, 1, sms);
     if (choose_msub(d.n, R, d.d_in, bn1) == 1) {
         GemmParams p = base_params(d.n, R, d.d_in, bn1, 1);
         const int S = small_launch_splits(p.m_tiles * p.n_tiles, p.k_blocks, sms);
@@ -172,7 +172,7 @@ int64_t fwd_part_elems(const cola_desc_t& d, int nproj, int sms)
             need = std::max<int64_t>(need, p.splits * partial_elems(p, bn1, 1));
         }
     }
-    const int bn2 = choose_bn_for(d.n, d.d_out, d.r);
+    const int bn2 = fill_bn(d.n, d.d_out, d.r, nproj, sms);
     if (choose_msub(d.n, d.d_out, d.r, bn2) == 1) {
         GemmParams p = base_params(d.n, d.d_out, d.r, bn2, 1);
         const int S = small_launch_splits(nproj * p.m_tiles * p.n_tiles, p.k_blocks, sms);
@@ -298,7 +298,7 @@ cola_status_t run_batch(int kind, int bn, int msub, const GemmProblem* probs, co
 // ------------------------------------------------------------ passes
 }  // namespace
 
-cudaError_t launch_splitk_cluster(const CredBatch& b, bool pdl, cudaStream_t stream);
+cudaError_t launch_splitk_cluster(const CredBatch& b, int op, int sigma, bool pdl, cudaStream_t stream);
 cudaError_t launch_thin(const ThinBatch& b, int kind, int sigma, cudaStream_t stream);
 
 namespace {
@@ -332,7 +332,6 @@ cola_status_t run_cluster_wgrad(int count, const CredJob* jobs, int64_t ntok, in
     b.count = count;
     b.S = S;
     b.kps = (kb + S - 1) / S;
-    b.op = accumulate_f32 ? CRED_ACC : CRED_STORE;
     b.status = status;
     int64_t mnk[MAX_GROUP][3];
     double flops = 0.0;
@@ -358,12 +357,11 @@ cola_status_t run_cluster_wgrad(int count, const CredJob* jobs, int64_t ntok, in
     }
     b.tiles = tiles;
     return launched(traced(COLA_KERNEL_WGRAD, count, mnk, S, TRACE_CLUSTER, st,
-                           [&] { return launch_splitk_cluster(b, flops < 64e9, st); }));
+                           [&] {
+                               return launch_splitk_cluster(b, accumulate_f32 ? CRED_ACC : CRED_STORE, SIG_IDENTITY,
+                                                            flops < 64e9, st);
+                           }));
 }
-
-// A reduce launch after a split weight-gradient launch, in k-block steps of
-// the busiest CTA (a few microseconds), for the comparison below.
-constexpr double REDUCE_LAUNCH_KB = 16.0;
 
 // The cluster split of a weight-gradient group (128 x 128 tiles, at most 8
 // splits, one wave of clusters): > 1 when it applies -- each CTA walks at
@@ -371,7 +369,7 @@ constexpr double REDUCE_LAUNCH_KB = 16.0;
 // planned schedule with its reduce launch.  Its 4-stage, one-tile-per-CTA
 // form is made for short token walks: at 65536 tokens (the LLaMA-60M block,
 // 128-171 k-blocks per CTA) it ran the weight gradients 60 -> 93 us.
-constexpr int CLUSTER_MAX_KPS = 16;
+constexpr int CLUSTER_MAX_KPS = 32;
 
 int wgrad_cluster_splits(const WgradPlan& w, int64_t ntok, int accumulate_f32, int sms)
 {
@@ -382,20 +380,89 @@ int wgrad_cluster_splits(const WgradPlan& w, int64_t ntok, int accumulate_f32, i
     const int kb = static_cast<int>((ntok + BK - 1) / BK);
     const int S = cluster_splits(tiles, kb, sms);
     if (S < 2 || (kb + S - 1) / S > CLUSTER_MAX_KPS) return 1;
-    double planned = w.cost + REDUCE_LAUNCH_KB;
+    double planned = w.cost;
     if (!accumulate_f32) {
         const TailPlan tp = wgrad_tail_plan(w, ntok, sms);
-        if (tail_wins(w, tp)) planned = tp.cost + (tp.pieces > 1 ? REDUCE_LAUNCH_KB : 0.0);
+        if (tail_wins(w, tp)) planned = tp.cost;
     }
     return (kb + S - 1) / S <= planned ? S : 1;
 }
+
+// One rank-r GEMM of few output tiles, D_j [n x N] for j < count over K, its K
+// splits reduced on clusters of S CTAs: Z, H (dY null: X A^T) or dZ, H
+// (dY_j B_j).
+struct RankGemm {
+    const void* T[3];         // token operand (X, dY_j), K-major
+    int64_t ldt;
+    const void* W[3];         // A [N x K] K-major, or B_j [K x N] (pitch N), read MN-major
+    int64_t ldw;
+    void* out[3];             // Z or null / dZ_j
+    void* out2[3];            // H / H_j or null
+    const void* zin[3];       // saved Z_j
+    int64_t ldo;
+};
+
+cola_status_t run_cluster_rank(int op, int sigma, int count, int64_t n, int64_t N, int64_t K, const RankGemm& g, int S,
+                               unsigned int* status, cudaStream_t st)
+{
+    CredBatch b;
+    std::memset(&b, 0, sizeof b);
+    const int kb = static_cast<int>((K + BK - 1) / BK);
+    b.count = count;
+    b.S = S;
+    b.kps = (kb + S - 1) / S;
+    b.status = status;
+    int64_t mnk[MAX_GROUP][3];
+    for (int j = 0; j < count; ++j) {
+        CredProblem& P = b.prob[j];
+        COLA_MAP(map_kmajor(&P.map_a, g.T[j], K, n, g.ldt, BM));
+        if (op == CRED_ZH)
+            COLA_MAP(map_kmajor(&P.map_b, g.W[j], K, N, g.ldw, CBN));
+        else
+            COLA_MAP(map_mnmajor(&P.map_b, g.W[j], N, K, g.ldw));
+        P.M = static_cast<int>(n);
+        P.N = static_cast<int>(N);
+        P.k_blocks = kb;
+        P.m_tiles = static_cast<int>((n + BM - 1) / BM);
+        P.n_tiles = static_cast<int>((N + CBN - 1) / CBN);
+        P.tile_begin = b.tiles;
+        b.tiles += P.m_tiles * P.n_tiles;
+        P.out = g.out[j];
+        P.out2 = static_cast<__nv_bfloat16*>(g.out2[j]);
+        P.zin = static_cast<const __nv_bfloat16*>(g.zin[j]);
+        P.ldo = g.ldo;
+        mnk[j][0] = n;
+        mnk[j][1] = N;
+        mnk[j][2] = K;
+    }
+    const bool zh = op == CRED_ZH;
+    const int flags = ((zh ? g.out[0] && g.out2[0] : g.out2[0] != nullptr) ? 1 : 0) | TRACE_CLUSTER;
+    return launched(traced(zh ? COLA_KERNEL_FWD_ZH : COLA_KERNEL_BWD_DZ, count, mnk, S, flags, st,
+                           [&] { return launch_splitk_cluster(b, op, sigma, true, st); }));
+}
+
+bool fused_fwd_form(const Shape& s, int sms);
+bool fused_bwd_form(const Shape& s, int sms);
 
 // F1: Z = X A^T, H = sigma(Z)  (N = r, or 3r for the fused q/k/v factors;
 // Z / H pitch ldz)
 cola_status_t run_f1(const Shape& s, int sigma, int64_t N, const void* X, const void* A, void* Z, void* H,
                      int64_t ldz, float* part, size_t part_bytes, unsigned int* status, int sms, cudaStream_t st)
 {
-    const int bn = choose_bn_for(s.n, N, s.d_in);
+    const int Sc = rank_gemm_splits(s.n, N, s.d_in, 1, sms);
+    // (a lone layer with the single-kernel form has to match it bit for bit)
+    if (Sc > 1 && g_cluster_splitk.load(std::memory_order_relaxed) && !(N == s.r && fused_fwd_form(s, sms))) {
+        RankGemm g = {};
+        g.T[0] = X;
+        g.ldt = s.ld_x;
+        g.W[0] = A;
+        g.ldw = s.ld_a;
+        g.out[0] = Z;
+        g.out2[0] = H;
+        g.ldo = ldz;
+        return run_cluster_rank(CRED_ZH, sigma, 1, s.n, N, s.d_in, g, Sc, status, st);
+    }
+    const int bn = fill_bn(s.n, N, s.d_in, 1, sms);
     const int ms = choose_msub(s.n, N, s.d_in, bn);
     GemmProblem pr;
     std::memset(&pr, 0, sizeof pr);
@@ -582,11 +649,16 @@ cola_status_t run_thin_glu(const Shape& s, const void* H_cat, const void* Bg, co
 // The single-kernel dZ + dX applies on the same terms: r = 64 or 128, at
 // most one 128-row tile per SM, neither GEMM compute-heavy (the backward's
 // GEMMs are never split over K).
-bool fused_bwd_applies(const Shape& s, int sms)
+bool fused_bwd_form(const Shape& s, int sms)
 {
-    if (!g_fused_bwd.load(std::memory_order_relaxed) || (s.r != 64 && s.r != 128)) return false;
+    if (s.r != 64 && s.r != 128) return false;
     if ((s.n + BM - 1) / BM > sms) return false;
     return !heavy_gemm(s.n, s.r, s.d_out) && !heavy_gemm(s.n, s.d_in, s.r);
+}
+
+bool fused_bwd_applies(const Shape& s, int sms)
+{
+    return g_fused_bwd.load(std::memory_order_relaxed) && fused_bwd_form(s, sms);
 }
 
 // Work items of a fused pass: the output blocks of a tile shared by up to
@@ -676,7 +748,7 @@ cola_status_t run_fused_bwd(const Shape& s, int sigma, const void* dY, const voi
 cola_status_t run_f2(const Shape& s, int count, const void* const* H, int64_t ldh, const void* const* B,
                      void* const* Y, float* part, size_t part_bytes, unsigned int* status, int sms, cudaStream_t st)
 {
-    const int bn = choose_bn_for(s.n, s.d_out, s.r);
+    const int bn = fill_bn(s.n, s.d_out, s.r, count, sms);
     const int ms = choose_msub(s.n, s.d_out, s.r, bn);
     GemmProblem pr[MAX_GROUP];
     int64_t mnk[MAX_GROUP][3];
@@ -748,7 +820,22 @@ cola_status_t run_b1(const Shape& s, int sigma, int count, const void* const* dY
                      const void* const* Z, int64_t ldz, void* const* dZ, void* const* Hout, unsigned int* status,
                      int sms, cudaStream_t st)
 {
-    const int bn = choose_bn_for(s.n, s.r, s.d_out);
+    const int Sc = rank_gemm_splits(s.n, s.r, s.d_out, count, sms);
+    if (Sc > 1 && g_cluster_splitk.load(std::memory_order_relaxed) && !(count == 1 && fused_bwd_form(s, sms))) {
+        RankGemm g = {};
+        g.ldt = s.ld_y;
+        g.ldw = s.r;
+        g.ldo = ldz;
+        for (int j = 0; j < count; ++j) {
+            g.T[j] = dY[j];
+            g.W[j] = B[j];
+            g.out[j] = dZ[j];
+            g.out2[j] = Hout ? Hout[j] : nullptr;
+            g.zin[j] = Z[j];
+        }
+        return run_cluster_rank(CRED_DZ, sigma, count, s.n, s.r, s.d_out, g, Sc, status, st);
+    }
+    const int bn = fill_bn(s.n, s.r, s.d_out, count, sms);
     const int ms = choose_msub(s.n, s.r, s.d_out, bn);
     GemmProblem pr[MAX_GROUP];
     int64_t mnk[MAX_GROUP][3];
@@ -1352,7 +1439,6 @@ cola_status_t cola_selftest_wait_timeout_cluster(void* ws, size_t ws_bytes, void
     b.tiles = 1;
     b.S = 2;
     b.kps = 4;
-    b.op = CRED_STORE;
     b.status = ws_status(ws);
     b.selftest = 1;
     CredProblem& P = b.prob[0];
@@ -1368,7 +1454,10 @@ cola_status_t cola_selftest_wait_timeout_cluster(void* ws, size_t ws_bytes, void
     P.ldo = N;
     const int64_t mnk[1][3] = {{M, N, T}};
     return launched(traced(COLA_KERNEL_WGRAD, 1, mnk, 2, TRACE_CLUSTER, static_cast<cudaStream_t>(stream),
-                           [&] { return launch_splitk_cluster(b, false, static_cast<cudaStream_t>(stream)); }));
+                           [&] {
+                               return launch_splitk_cluster(b, CRED_STORE, SIG_IDENTITY, false,
+                                                            static_cast<cudaStream_t>(stream));
+                           }));
 }
 
 cola_status_t cola_check_status(void* ws, void* stream, uint32_t* code_out)

@@ -1095,7 +1095,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         int zu = first_unit, zc = c_first;      // next item whose boxes are to be loaded
         uint32_t zphase = 0;                    // bit b: parity of the next wait on zbar[b]
         int zload = 0, zuse = 0;                // items loaded, items used: item i in slot i % ZSLOTS
-        int zslot_l = 0, zslot_u = 0;
+        int zslot_l = 0, zslot_u = 0;           // i % ZSLOTS, where that is not i & 1
         int zsub = 0;                           // GLU_ONE: 0 = Y_up is next, 1 = Y_gate
         auto z_advance = [&]() {                // move (zu, zc) to the next item that has a chunk
             while (zu < batch.units && zc >= chunk_count(decode(batch, zu))) {
@@ -1106,7 +1106,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         auto z_issue = [&]() {                  // load the boxes of item (zu, zc), then step past it
             if (zu >= batch.units) return;
             const Unit x = decode(batch, zu);
-            const int b = zslot_l;
+            const int b = ZSLOTS == 2 ? zload & 1 : zslot_l;
             if (lane == 0) {
                 bulk_wait_group_read<0>();      // the stores that last read slot b are done with it
                 const int xc = x.n_blk * BN + zc * CHUNK, yr = x.m_blk * TILE_M + row_off + sub * BM + q * 32;
@@ -1123,7 +1123,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 }
             }
             ++zload;
-            if (++zslot_l == ZSLOTS) zslot_l = 0;
+            if (ZSLOTS != 2 && ++zslot_l == ZSLOTS) zslot_l = 0;
             if (GLU_ONE && zsub == 0) {
                 zsub = 1;
                 return;
@@ -1346,11 +1346,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     if (!GLU_ONE) z_issue();   // the next chunk's boxes, into the slot stored from a chunk ago
 #pragma unroll 1
                     for (int f = 0; f < (GLU_ONE ? 2 : 1); ++f) {
-                        const int b = zslot_u;
+                        const int b = ZSLOTS == 2 ? zuse & 1 : zslot_u;
                         ok = wait_bounded(&zbar[b], (zphase >> b) & 1u, wc, ST_TIMEOUT_EPILOGUE);
                         zphase ^= 1u << b;
                         ++zuse;
-                        if (++zslot_u == ZSLOTS) zslot_u = 0;
+                        if (ZSLOTS != 2 && ++zslot_u == ZSLOTS) zslot_u = 0;
                         if (!ok) break;
                         const uint32_t box = ep + b * epi_slot_bytes(EPI);
                         times_dm(box, f == 0 ? p.d_ptr : p.d2_ptr);
@@ -1434,11 +1434,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         emit(p.h_only ? map_d : map_d2, w, col0, row0);
                     }
                 } else if (DSIG) {
-                    const int b = zslot_u;
+                    const int b = ZSLOTS == 2 ? zuse & 1 : zslot_u;
                     const bool zok = wait_bounded(&zbar[b], (zphase >> b) & 1u, wc, ST_TIMEOUT_EPILOGUE);
                     zphase ^= 1u << b;
                     ++zuse;
-                    if (++zslot_u == ZSLOTS) zslot_u = 0;
+                    if (ZSLOTS != 2 && ++zslot_u == ZSLOTS) zslot_u = 0;
                     if (!zok) {
                         ok = false;
                         break;
@@ -1513,7 +1513,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         }
         // Z boxes still in flight (issued ahead, or for items the loop left early)
         while (zuse < zload) {
-            const int b = zslot_u;
+            const int b = ZSLOTS == 2 ? zuse & 1 : zslot_u;
             const uint64_t t0 = global_timer_ns();
             while (!mbar_try_wait(&zbar[b], (zphase >> b) & 1u)) {
                 if (global_timer_ns() - t0 > WAIT_LIMIT_NS) {
@@ -1523,7 +1523,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             }
             zphase ^= 1u << b;
             ++zuse;
-            if (++zslot_u == ZSLOTS) zslot_u = 0;
+            if (ZSLOTS != 2 && ++zslot_u == ZSLOTS) zslot_u = 0;
         }
         if (lane == 0) bulk_wait_group_all();   // every output store has landed
     }

@@ -1,5 +1,4 @@
-// The cluster-reduced split-K GEMM (splitk_cluster.cuh): its launcher, for
-// the weight gradients (token-major, MN-major operands).
+// The cluster-reduced split-K GEMMs (splitk_cluster.cuh): their launcher.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -9,11 +8,14 @@
 
 namespace cola {
 
-cudaError_t launch_splitk_cluster(const CredBatch& b, bool pdl, cudaStream_t stream)
+namespace {
+
+template <bool A_MN, bool B_MN, int OP, int SIG>
+cudaError_t launch_one(const CredBatch& b, bool pdl, cudaStream_t stream)
 {
-    if (b.S < 1 || b.S > MAX_CLUSTER || b.tiles < 1) return cudaErrorInvalidValue;
+    if (b.S < (OP == CRED_DZ ? 2 : 1) || b.S > MAX_CLUSTER || b.tiles < 1) return cudaErrorInvalidValue;
     constexpr int smem = CredCfg::SMEM_BYTES;
-    auto kern = splitk_cluster_kernel;
+    auto kern = splitk_cluster_kernel<A_MN, B_MN, OP, SIG>;
     static std::atomic<unsigned long long> configured{0};   // bit d: attribute set on device d
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -25,7 +27,7 @@ cudaError_t launch_splitk_cluster(const CredBatch& b, bool pdl, cudaStream_t str
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(b.tiles * b.S));
-    cfg.blockDim = dim3(NUM_THREADS);
+    cfg.blockDim = dim3(CRED_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -38,6 +40,28 @@ cudaError_t launch_splitk_cluster(const CredBatch& b, bool pdl, cudaStream_t str
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kern, b);
+}
+
+}  // namespace
+
+cudaError_t launch_splitk_cluster(const CredBatch& b, int op, int sigma, bool pdl, cudaStream_t stream)
+{
+    if (op == CRED_STORE) return launch_one<true, true, CRED_STORE, SIG_IDENTITY>(b, pdl, stream);
+    if (op == CRED_ACC) return launch_one<true, true, CRED_ACC, SIG_IDENTITY>(b, pdl, stream);
+    const bool zh = op == CRED_ZH;
+    if (!zh && op != CRED_DZ) return cudaErrorInvalidValue;
+    switch (sigma) {
+    case SIG_SILU:
+        return zh ? launch_one<false, false, CRED_ZH, SIG_SILU>(b, pdl, stream)
+                  : launch_one<false, true, CRED_DZ, SIG_SILU>(b, pdl, stream);
+    case SIG_GELU:
+        return zh ? launch_one<false, false, CRED_ZH, SIG_GELU>(b, pdl, stream)
+                  : launch_one<false, true, CRED_DZ, SIG_GELU>(b, pdl, stream);
+    case SIG_IDENTITY:
+        return zh ? launch_one<false, false, CRED_ZH, SIG_IDENTITY>(b, pdl, stream)
+                  : launch_one<false, true, CRED_DZ, SIG_IDENTITY>(b, pdl, stream);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace cola

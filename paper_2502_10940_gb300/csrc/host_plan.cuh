@@ -117,6 +117,15 @@ int choose_bn_for(int64_t M, int64_t N, int64_t K)
     return choose_bn(N, heavy_gemm(M, N, K));
 }
 
+// The same for `count` GEMMs of one launch, with 128 columns where those tiles
+// still run in one wave: twice the CTAs of 256-column ones.
+int fill_bn(int64_t M, int64_t N, int64_t K, int count, int sms)
+{
+    const int bn = choose_bn_for(M, N, K);
+    if (bn == 128 || heavy_gemm(M, N, K)) return bn;
+    return count * ((M + BM - 1) / BM) * ((N + 127) / 128) <= sms ? 128 : 256;
+}
+
 // Tile modes ("msub" below): 1 = one CTA runs a 128-row tile; 2 = one CTA
 // runs two 128-row sub-tiles sharing each B tile; TILE_PAIR = a CTA pair runs
 // a 256-row tile with tcgen05 cta_group::2 (each CTA loads half of B).
@@ -158,6 +167,10 @@ GemmParams base_params(int64_t M, int64_t N, int64_t K, int bn, int msub)
     p.units = p.m_tiles * p.n_tiles;
     return p;
 }
+
+// A reduce launch after a split weight-gradient launch, in k-block steps of
+// the busiest CTA (a few microseconds).
+constexpr double REDUCE_LAUNCH_KB = 16.0;
 
 // Token split of weight-gradient GEMMs sharing one launch (same K): minimise
 // (waves of persistent CTAs) x (k-blocks per unit + the cost of writing and
@@ -212,11 +225,26 @@ int small_launch_splits(int tiles, int k_blocks, int sms)
 // per split.  1 = no split.
 int cluster_splits(int tiles, int k_blocks, int sms)
 {
-    if (tiles < 1 || 2 * tiles >= sms) return 1;
+    if (tiles < 1 || 2 * tiles > sms) return 1;
     int s = sms / tiles;
     if (s > MAX_CLUSTER) s = MAX_CLUSTER;
     if (s > k_blocks / 4) s = k_blocks / 4;
     return s < 1 ? 1 : s;
+}
+
+// K splits, inside clusters, of the `count` rank-r GEMMs of one launch (Z of the
+// forward, dZ of the backward): 128 x 128 tiles, fewer than half the SMs, not
+// compute-heavy.  1 = no split.  Measured against fp32 slabs with a reduce launch
+// (Z) and an unsplit dZ, whole graph-replayed passes with the schedules below:
+// q/k/v of 509 tokens, d = 1024, r = 256 23.9 -> 16.4 us forward, 58.8 -> 37.4 us
+// with its backward; a 150-token layer 3000 -> 3000, r = 768 66.1 -> 41.1 us; a
+// 2048-token 350M-shaped block 268 -> 192 us.
+int rank_gemm_splits(int64_t n, int64_t N, int64_t K, int count, int sms)
+{
+    if (heavy_gemm(n, N, K)) return 1;
+    const int64_t tiles = count * ((n + BM - 1) / BM) * ((N + CBN - 1) / CBN);
+    if (2 * tiles > sms) return 1;
+    return cluster_splits(static_cast<int>(tiles), static_cast<int>((K + BK - 1) / BK), sms);
 }
 
 // Split of a thin launch (thin.cuh): `tiles` 128-row weight tiles over k_blocks
@@ -274,6 +302,11 @@ WgradPlan plan_wgrad(const int64_t* M, const int64_t* N, int count, int64_t ntok
         const int ms = choose_msub(M[i], N[i], ntok, w.bn);
         if (ms == 1 || (ms == 2 && w.msub == TILE_PAIR)) w.msub = ms;
     }
+    if (w.bn == 256 && w.msub == 1) {   // 128 columns where those tiles still run in one wave
+        int64_t t = 0;
+        for (int i = 0; i < count; ++i) t += ((M[i] + BM - 1) / BM) * ((N[i] + 127) / 128);
+        if (t <= sms) w.bn = 128;
+    }
     int tiles = 0;
     for (int i = 0; i < count; ++i) {
         w.p[i] = base_params(M[i], N[i], ntok, w.bn, w.msub);
@@ -296,7 +329,7 @@ WgradPlan plan_wgrad(const int64_t* M, const int64_t* N, int count, int64_t ntok
         const int sl = unit_slots(w.msub, sms);
         const long long units = static_cast<long long>(tiles) * w.splits;
         const long long waves = (units + sl - 1) / sl;
-        w.cost = static_cast<double>(waves) * (w.p[0].kb_per_split + (w.splits > 1 ? c_part : 0.0));
+        w.cost = static_cast<double>(waves) * (w.p[0].kb_per_split + (w.splits > 1 ? c_part : 0.0)) + REDUCE_LAUNCH_KB;
     }
     return w;
 }
@@ -342,6 +375,8 @@ TailPlan plan_tail(const GemmParams* p, int count, int bn, int msub, int sms)
     s.tail = R;
     s.pieces = 1;
     s.kps = s.kb;
+    const int rows = tile_rows(msub);
+    const double c_part = 8.0 * bn * rows / (128.0 * (rows + bn)) + 2.0;   // as in choose_splits
     if (R > 0 && R <= MAX_TAIL_TILES) {
         const int most = s.kb / 4 > 1 ? s.kb / 4 : 1;
         int St = slots / R < most ? slots / R : most;
@@ -349,13 +384,12 @@ TailPlan plan_tail(const GemmParams* p, int count, int bn, int msub, int sms)
             s.kps = (s.kb + St - 1) / St;
             St = (s.kb + s.kps - 1) / s.kps;   // no empty piece
         }
-        s.pieces = St > 1 ? St : 1;
+        // the pieces' partials and the reduce launch have to pay for themselves
+        s.pieces = St > 1 && s.kps + c_part + REDUCE_LAUNCH_KB < s.kb ? St : 1;
         if (s.pieces == 1) s.kps = s.kb;
     }
     s.units = s.body + R * s.pieces;
-    const int rows = tile_rows(msub);
-    const double c_part = 8.0 * bn * rows / (128.0 * (rows + bn)) + 2.0;   // as in choose_splits
-    s.cost = static_cast<double>(waves) * s.kb + (R > 0 ? s.kps + (s.pieces > 1 ? c_part : 0.0) : 0.0);
+    s.cost = static_cast<double>(waves) * s.kb + (R > 0 ? s.kps + (s.pieces > 1 ? c_part + REDUCE_LAUNCH_KB : 0.0) : 0.0);
     if (s.pieces > 1) {
         s.part_elems = static_cast<int64_t>(R) * s.pieces * rows * bn;
         s.ntiles = R;

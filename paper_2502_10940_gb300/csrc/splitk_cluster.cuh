@@ -1,10 +1,12 @@
-// splitk_cluster.cuh -- weight gradients whose token splits are reduced
-// inside a thread-block cluster (sm_103a), for launches with few output tiles
-// (a few thousand tokens):
+// splitk_cluster.cuh -- GEMMs of few output tiles whose K splits are reduced
+// inside a thread-block cluster (sm_103a), for launches of a few thousand
+// tokens:
 //
-//   D[tile] = sum over s = 0..S-1 of  sum over tokens t of split s of  P[t, m] Q[t, n]
+//   D[tile] = sum over s = 0..S-1 of  sum over k of split s of  P[m, k] Q[n, k]
 //
-// (dB = dY^T H, dA = dZ^T X, Sec. 3.4; P and Q token-major, read MN-major.)
+// the weight gradients (dB = dY^T H, dA = dZ^T X, Sec. 3.4: k = tokens, P and Q
+// token-major, read MN-major), Z = X A^T with H = sigma(Z) (both K-major),
+// dZ = (dY B) * sigma'(Z) (B read MN-major) and Y = H B^T (both K-major).
 //
 // Each 128 x 128 output tile runs on one cluster of S CTAs (1 <= S <= 8),
 // CTA s accumulating the k-blocks of split s in its own TMEM.  The partial
@@ -22,11 +24,11 @@
 // (j xor (row mod 8)): the writes of 32 rows are free of bank conflicts, and
 // the owner reads the rows back in order.
 //
-// Epilogues (CredOp): a bf16 store, or an fp32 accumulate (D += sum, for
-// gradients accumulated in fp32).  The forward GEMMs of a handful of tokens
-// were run this way too, and measured no faster than their slab split with
-// a reduce launch (which overlaps the GEMM's tail): 1B-shaped 32-token
-// forward 0.0659 against 0.0661 ms, 7B-shaped 0.093 against 0.091 ms.
+// Epilogues (CredOp), on the summed rows: a bf16 store, an fp32 accumulate
+// (D += sum, for gradients accumulated in fp32), Z and H = sigma(Z), or
+// dZ = sum * sigma'(Z) (and H) with the saved Z read ahead of the exchange.
+// Against fp32 slabs with a reduce launch (Z, H) and an unsplit dZ: see
+// rank_gemm_splits (host_plan.cuh).
 //
 // The receive buffer (S bands of up to ceil(128 / S) rows, at most 133 rows
 // of 128 fp32) has shared memory of its own,
@@ -46,9 +48,9 @@
 // against 2 s), so that the bands of a CTA that gave up still land before
 // anyone exits.
 //
-// Warp roles as in gemm.cuh (320 threads, one CTA per SM): warp 0 TMA
-// producer, warp 1 MMA issuer (allocates TMEM), warps 2..9 the exchange and
-// the reduction.
+// Warp roles (576 threads, one CTA per SM): warp 0 TMA producer, warp 1 MMA
+// issuer (allocates TMEM), warps 2..17 the exchange and the reduction, whose
+// sums and activations are chains that more warps hide.
 #pragma once
 #include "gemm.cuh"
 
@@ -93,21 +95,28 @@ __device__ __forceinline__ bool exchange_wait(uint64_t* bar, uint64_t limit, uns
     return true;
 }
 
-// Named barrier of the eight exchange warps.
-__device__ __forceinline__ void exchange_warps_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
-enum CredOp : int { CRED_STORE = 0, CRED_ACC = 1 };
+
+enum CredOp : int { CRED_STORE = 0, CRED_ACC = 1, CRED_ZH = 2, CRED_DZ = 3 };
 
 constexpr int CBN = 128;        // tile width
+constexpr int CRED_WARPS = 16;  // exchange and reduction warps, four per TMEM lane quarter
+constexpr int CRED_THREADS = 64 + 32 * CRED_WARPS;
+static_assert(CRED_WARPS == 4 * (CBN / 32), "one 32-column chunk per warp");
 constexpr int MAX_CLUSTER = 8;  // portable cluster size
+
+// Named barrier of the exchange warps.
+__device__ __forceinline__ void exchange_warps_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * CRED_WARPS) : "memory"); }
 
 struct CredProblem {
     CUtensorMap map_a, map_b;
     int M, N, k_blocks;
     int m_tiles, n_tiles;
     int tile_begin;   // first batch-wide tile of this problem
-    void* out;        // CRED_STORE: bf16 D; CRED_ACC: fp32 D
-    long long ldo;    // row pitch of out, elements
+    void* out;        // CRED_STORE: bf16 D; CRED_ACC: fp32 D; CRED_ZH: Z or null; CRED_DZ: dZ
+    long long ldo;    // row pitch of out (and out2, zin), elements
+    __nv_bfloat16* out2;        // CRED_ZH: H; CRED_DZ: H or null
+    const __nv_bfloat16* zin;   // CRED_DZ: the saved Z
 };
 
 // Up to MAX_GROUP GEMMs with the same K, their tiles numbered problem after
@@ -119,7 +128,6 @@ struct CredBatch {
     int tiles;
     int S;      // CTAs per cluster = K splits, 1 ... MAX_CLUSTER
     int kps;    // k-blocks per split (the last split may have fewer, or none)
-    int op;     // CredOp
     unsigned int* status;
     // failure-detection self-test: 1 = CTA rank 1 of the first cluster issues
     // no loads, so its MMA issuer's first wait runs out while the other CTAs
@@ -143,7 +151,9 @@ struct CredCfg {
 // The kernel itself is compiled in one translation unit (gemm_cluster.cu);
 // the others see the batch description only.
 #ifdef COLA_DEFINE_CLUSTER_KERNEL
-__global__ void __launch_bounds__(NUM_THREADS, 1) splitk_cluster_kernel(const __grid_constant__ CredBatch b)
+// A_MN / B_MN: the operand is MN-major (token-major, read transposed).
+template <bool A_MN, bool B_MN, int OP, int SIG>
+__global__ void __launch_bounds__(CRED_THREADS, 1) splitk_cluster_kernel(const __grid_constant__ CredBatch b)
 {
     using C = CredCfg;
     constexpr int STAGES = C::STAGES;
@@ -228,11 +238,22 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) splitk_cluster_kernel(const __
                 uint8_t* sa = smem_a + stage * C::A_BYTES;
                 uint8_t* sb = smem_b + stage * C::B_BYTES;
                 mbar_arrive_expect_tx(&full_bar[stage], C::STAGE_BYTES);
-                // MN-major operands: 64-column boxes along M (N), 64 tokens deep
+                // MN-major operands: 64-column boxes along M (N), 64 k deep; K-major
+                // ones: one box of 128 rows
+                if (A_MN) {
 #pragma unroll
-                for (int j = 0; j < BM / 64; ++j) tma_load_2d(&P.map_a, &full_bar[stage], sa + j * 64 * BK * 2, m0 + 64 * j, kb * BK);
+                    for (int j = 0; j < BM / 64; ++j)
+                        tma_load_2d(&P.map_a, &full_bar[stage], sa + j * 64 * BK * 2, m0 + 64 * j, kb * BK);
+                } else {
+                    tma_load_2d(&P.map_a, &full_bar[stage], sa, kb * BK, m0);
+                }
+                if (B_MN) {
 #pragma unroll
-                for (int j = 0; j < CBN / 64; ++j) tma_load_2d(&P.map_b, &full_bar[stage], sb + j * 64 * BK * 2, n0 + 64 * j, kb * BK);
+                    for (int j = 0; j < CBN / 64; ++j)
+                        tma_load_2d(&P.map_b, &full_bar[stage], sb + j * 64 * BK * 2, n0 + 64 * j, kb * BK);
+                } else {
+                    tma_load_2d(&P.map_b, &full_bar[stage], sb, kb * BK, n0);
+                }
                 ++issued;
                 if (++stage == STAGES) {
                     stage = 0;
@@ -276,7 +297,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) splitk_cluster_kernel(const __
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
         if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16_f32(BM, CBN, 1, 1);
+            constexpr uint32_t idesc = idesc_bf16_f32(BM, CBN, A_MN ? 1 : 0, B_MN ? 1 : 0);
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true, issued_any = false;
@@ -290,9 +311,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) splitk_cluster_kernel(const __
                 const uint32_t sb = smem_u32(smem_b + stage * C::B_BYTES);
 #pragma unroll
                 for (int ks = 0; ks < BK / UMMA_K; ++ks) {
-                    // next 16 tokens: +16 rows of 128 bytes; 64-column groups 8 KB apart
-                    const uint64_t da = smem_desc_sw128(sa + ks * UMMA_K * 128, 64 * BK * 2, 1024);
-                    const uint64_t db = smem_desc_sw128(sb + ks * UMMA_K * 128, 64 * BK * 2, 1024);
+                    // next 16 k: +16 rows of 128 bytes (MN-major, 64-column groups 8 KB
+                    // apart) or +32 bytes inside the swizzled row (K-major)
+                    const uint64_t da = A_MN ? smem_desc_sw128(sa + ks * UMMA_K * 128, 64 * BK * 2, 1024)
+                                             : smem_desc_sw128(sa + ks * UMMA_K * 2, 16, 1024);
+                    const uint64_t db = B_MN ? smem_desc_sw128(sb + ks * UMMA_K * 128, 64 * BK * 2, 1024)
+                                             : smem_desc_sw128(sb + ks * UMMA_K * 2, 16, 1024);
                     umma_f16(tmem_base, da, db, idesc, (kb > kb0 || ks > 0) ? 1u : 0u);
                 }
                 issued_any = true;
@@ -316,10 +340,26 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) splitk_cluster_kernel(const __
             }
         }
     } else {
-        // ------------------------------------------------ exchange and reduction (warps 2..9)
+        // ------------------------------------------------ exchange and reduction (warps 2..17)
         const int q = warp & 3;                 // TMEM lane quarter
-        const int half = (warp - 2) >> 2;       // alternate 32-column chunks
+        const int c = (warp - 2) >> 2;          // this warp's 32-column chunk
         const int row = q * 32 + lane;          // this thread's row of the partial tile
+        const int tid = threadIdx.x - 64;
+        const int items = my_rows * (CBN / 4);   // groups of 4 columns of this CTA's band
+        // CRED_DZ: this thread's groups of the saved Z, loaded ahead of the exchange
+        constexpr int ZGROUPS = OP == CRED_DZ ? (BM / 2) * (CBN / 4) / (CRED_WARPS * 32) : 1;   // S >= 2
+        uint2 zg[ZGROUPS];
+        if (OP == CRED_DZ) {
+#pragma unroll
+            for (int i = 0; i < ZGROUPS; ++i) {
+                const int it = tid + i * CRED_WARPS * 32;
+                const int gr = m_blk * BM + static_cast<int>(rank) * RP + it / (CBN / 4);
+                const int gc = n_blk * CBN + (it % (CBN / 4)) * 4;
+                zg[i] = make_uint2(0u, 0u);
+                if (it < items && gr < P.M && gc < P.N)
+                    zg[i] = __ldg(reinterpret_cast<const uint2*>(P.zin + static_cast<long long>(gr) * P.ldo + gc));
+            }
+        }
         const bool acc_ok = wait_bounded(tfull, 0, wc, ST_TIMEOUT_EPILOGUE);
         tc_fence_after();
         // stage this row's partial in the ring: row-major fp32, 16-byte chunk j
@@ -327,9 +367,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) splitk_cluster_kernel(const __
         const uint32_t stg = smem_u32(smem) + static_cast<uint32_t>(row * CBN * 4);
         // an accumulator this CTA gave up on sends zeros (tcgen05.ld is warp-wide)
         const bool use_acc = __all_sync(0xffffffffu, acc_ok && has_k && !*abort_flag);
-#pragma unroll
-        for (int i = 0; i < CBN / 64; ++i) {
-            const int c = half + 2 * i;
+        {
             uint32_t v[32];
             if (use_acc) {
                 tmem_ld_32x32b_x32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(c * 32), v);
@@ -346,7 +384,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) splitk_cluster_kernel(const __
         tc_fence_before();
         fence_proxy_async_smem();   // the staged rows visible to the copy engine
         exchange_warps_sync();
-        const int tid = threadIdx.x - 64;
         if (tid < S) {
             // band `tid` of this partial into slot `rank` of its owner (slots of band_rows(tid) rows)
             const uint32_t bytes = static_cast<uint32_t>(band_rows(tid) * CBN * 4);
@@ -360,8 +397,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) splitk_cluster_kernel(const __
         // here has been read
         if (tid < S) mbar_arrive_cluster_relaxed(mapa_shared(smem_u32(done), static_cast<uint32_t>(tid)));
         if (dok && !*abort_flag) {
-            const int items = my_rows * (CBN / 4);
-            for (int it = tid; it < items; it += NUM_EPI_WARPS * 32) {
+            auto group = [&](int it, const uint2 z) {
                 const int lr = it / (CBN / 4), c4 = it - lr * (CBN / 4);
                 // slot s, row lr: row rank * RP + lr of every sender's staging
                 const int pos = (c4 ^ ((static_cast<int>(rank) * RP + lr) & 7)) * 4;
@@ -375,17 +411,33 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) splitk_cluster_kernel(const __
                 }
                 const int gr = m_blk * BM + static_cast<int>(rank) * RP + lr;
                 const int gc = n_blk * CBN + c4 * 4;
-                if (gr >= P.M || gc >= P.N) continue;
+                if (gr >= P.M || gc >= P.N) return;
                 const int valid = min(4, P.N - gc);
-                const float v[4] = {a.x, a.y, a.z, a.w};
                 const long long off = static_cast<long long>(gr) * P.ldo + gc;
-                if (b.op == CRED_ACC) {
+                if (OP == CRED_ACC) {
+                    const float v[4] = {a.x, a.y, a.z, a.w};
                     float* o = static_cast<float*>(P.out) + off;
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
                         if (e < valid) o[e] += v[e];
+                } else if (OP == CRED_ZH) {      // N is a multiple of 64: whole groups, 8-byte aligned
+                    const uint32_t z01 = pack_bf16x2(a.x, a.y), z23 = pack_bf16x2(a.z, a.w);
+                    if (P.out) *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(P.out) + off) = make_uint2(z01, z23);
+                    *reinterpret_cast<uint2*>(P.out2 + off) =
+                        make_uint2(pack_bf16x2(act_sigma<SIG>(bf16_lo(z01)), act_sigma<SIG>(bf16_hi(z01))),
+                                   pack_bf16x2(act_sigma<SIG>(bf16_lo(z23)), act_sigma<SIG>(bf16_hi(z23))));
+                } else if (OP == CRED_DZ) {
+                    float h[4], d[4];
+                    act_both<SIG>(bf16_lo(z.x), h[0], d[0]);
+                    act_both<SIG>(bf16_hi(z.x), h[1], d[1]);
+                    act_both<SIG>(bf16_lo(z.y), h[2], d[2]);
+                    act_both<SIG>(bf16_hi(z.y), h[3], d[3]);
+                    *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(P.out) + off) =
+                        make_uint2(pack_bf16x2(a.x * d[0], a.y * d[1]), pack_bf16x2(a.z * d[2], a.w * d[3]));
+                    if (P.out2)
+                        *reinterpret_cast<uint2*>(P.out2 + off) = make_uint2(pack_bf16x2(h[0], h[1]), pack_bf16x2(h[2], h[3]));
                 } else {
-                    const uint32_t w0 = pack_bf16x2(v[0], v[1]), w1 = pack_bf16x2(v[2], v[3]);
+                    const uint32_t w0 = pack_bf16x2(a.x, a.y), w1 = pack_bf16x2(a.z, a.w);
                     __nv_bfloat16* o = static_cast<__nv_bfloat16*>(P.out) + off;
                     if (valid == 4 && (reinterpret_cast<uintptr_t>(o) & 7) == 0) {
                         *reinterpret_cast<uint2*>(o) = make_uint2(w0, w1);
@@ -397,6 +449,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) splitk_cluster_kernel(const __
                             if (e < valid) o16[e] = static_cast<uint16_t>((e & 1) ? (w[e >> 1] >> 16) : (w[e >> 1] & 0xFFFFu));
                     }
                 }
+            };
+            if (OP == CRED_DZ) {
+#pragma unroll
+                for (int i = 0; i < ZGROUPS; ++i)
+                    if (tid + i * CRED_WARPS * 32 < items) group(tid + i * CRED_WARPS * 32, zg[i]);
+            } else {
+#pragma unroll 1
+                for (int it = tid; it < items; it += CRED_WARPS * 32) group(it, make_uint2(0u, 0u));
             }
         }
         // the bands this CTA sent have been read by their owners: its staging
