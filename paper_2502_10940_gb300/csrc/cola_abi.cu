@@ -1064,13 +1064,8 @@ cola_status_t run_b4_glu(const Shape& s, int64_t K, const void* dZ, int64_t ldz,
 cola_status_t run_b4(const Shape& s, int64_t K, const void* dZ, int64_t ldz, const void* A, void* dX,
                      unsigned int* status, int sms, cudaStream_t st)
 {
-    // CTA pairs where the plain dX GEMM takes them; otherwise 128 x 128 tiles
-    // (256-column ones would leave two operand stages beside the slots of
-    // Y_gate and Y_up boxes)
-    const int bn_x = choose_bn_for(s.n, s.d_in, K);
-    const bool pair = choose_msub(s.n, s.d_in, K, bn_x) == TILE_PAIR;
-    const int bn = pair ? 256 : 128;
-    const int ms = pair ? TILE_PAIR : 1;
+    const int bn = fill_bn(s.n, s.d_in, K, 1, sms);
+    const int ms = choose_msub(s.n, s.d_in, K, bn);
     GemmProblem pr;
     std::memset(&pr, 0, sizeof pr);
     pr.p = base_params(s.n, s.d_in, K, bn, ms);
