@@ -798,11 +798,12 @@ cola_status_t run_f2(const Shape& s, int count, const void* const* H, int64_t ld
                                    [&] { return launch_splitk_reduce(rb, st); }));
         }
     }
+    const bool wide = store_boxes64(ms == TILE_PAIR, s.ld_y, count * s.n * s.d_out * 2);
     for (int j = 0; j < count; ++j) {
         pr[j].p = base_params(s.n, s.d_out, s.r, bn, ms);
         COLA_MAP(map_kmajor(&pr[j].map_a, H[j], s.r, s.n, ldh, a_box_rows(ms)));
         COLA_MAP(map_kmajor(&pr[j].map_b, B[j], s.r, s.d_out, s.r, b_box_rows(bn, ms)));
-        COLA_MAP(map_box32(&pr[j].map_d, Y[j], s.d_out, s.n, s.ld_y));
+        COLA_MAP((wide ? map_box64 : map_box32)(&pr[j].map_d, Y[j], s.d_out, s.n, s.ld_y));
         pr[j].map_d2 = pr[j].map_z = pr[j].map_d;
         pr[j].p.d_ptr = static_cast<__nv_bfloat16*>(Y[j]);
         pr[j].p.d_ld = s.ld_y;
@@ -811,6 +812,8 @@ cola_status_t run_f2(const Shape& s, int count, const void* const* H, int64_t ld
         mnk[j][1] = s.d_out;
         mnk[j][2] = s.r;
     }
+    if (wide && ms != TILE_PAIR)
+        return run_batch<false, false, EPI_STORE64>(COLA_KERNEL_FWD_Y, bn, ms, pr, mnk, count, 0, sms, st);
     return run_batch<false, false, EPI_STORE>(COLA_KERNEL_FWD_Y, bn, ms, pr, mnk, count, 0, sms, st);
 }
 
@@ -1066,17 +1069,20 @@ cola_status_t run_b4(const Shape& s, int64_t K, const void* dZ, int64_t ldz, con
 {
     const int bn = fill_bn(s.n, s.d_in, K, 1, sms);
     const int ms = choose_msub(s.n, s.d_in, K, bn);
+    const bool wide = store_boxes64(ms == TILE_PAIR, s.ld_x, s.n * s.d_in * 2);
     GemmProblem pr;
     std::memset(&pr, 0, sizeof pr);
     pr.p = base_params(s.n, s.d_in, K, bn, ms);
     COLA_MAP(map_kmajor(&pr.map_a, dZ, K, s.n, ldz, a_box_rows(ms)));
     COLA_MAP(map_mnmajor(&pr.map_b, A, s.d_in, K, s.ld_a));
-    COLA_MAP(map_box32(&pr.map_d, dX, s.d_in, s.n, s.ld_x));
+    COLA_MAP((wide ? map_box64 : map_box32)(&pr.map_d, dX, s.d_in, s.n, s.ld_x));
     pr.map_d2 = pr.map_z = pr.map_d;
     pr.p.d_ptr = static_cast<__nv_bfloat16*>(dX);
     pr.p.d_ld = s.ld_x;
     pr.p.status = status;
     const int64_t mnk[1][3] = {{s.n, s.d_in, K}};
+    if (wide && ms != TILE_PAIR)
+        return run_batch<false, true, EPI_STORE64>(COLA_KERNEL_BWD_DX, bn, ms, &pr, mnk, 1, 0, sms, st);
     return run_batch<false, true, EPI_STORE>(COLA_KERNEL_BWD_DX, bn, ms, &pr, mnk, 1, 0, sms, st);
 }
 
@@ -1409,7 +1415,7 @@ cola_status_t cola_selftest_wait_timeout_pair(void* ws, size_t ws_bytes, int32_t
     pr.p = base_params(M, N, K, 256, TILE_PAIR);
     COLA_MAP(map_kmajor(&pr.map_a, base, K, M, K, a_box_rows(TILE_PAIR)));
     COLA_MAP(map_kmajor(&pr.map_b, base + a_bytes, K, N, K, b_box_rows(256, TILE_PAIR)));
-    COLA_MAP(map_box32(&pr.map_d, base + a_bytes + b_bytes, N, M, N));
+    COLA_MAP(map_box64(&pr.map_d, base + a_bytes + b_bytes, N, M, N));
     pr.map_d2 = pr.map_z = pr.map_d;
     pr.p.d_ptr = reinterpret_cast<__nv_bfloat16*>(base + a_bytes + b_bytes);
     pr.p.d_ld = N;

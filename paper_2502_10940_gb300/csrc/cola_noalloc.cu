@@ -105,7 +105,7 @@ extern "C" cola_status_t cola_wgrad_static_scratch(int64_t n_tokens, int64_t M, 
     pr.p.status = nullptr;   // no workspace to report a device-side timeout through
     if (pr.p.splits == 1 && !accumulate_f32) {
         // unsplit: the epilogue stores the bf16 gradient directly; no scratch
-        if (!map_box32(&pr.map_d, D, N, M, ld_d)) return COLA_ERR_LAUNCH;
+        if (!(w.msub == TILE_PAIR ? map_box64 : map_box32)(&pr.map_d, D, N, M, ld_d)) return COLA_ERR_LAUNCH;
         pr.map_d2 = pr.map_z = pr.map_d;
         pr.p.d_ptr = static_cast<__nv_bfloat16*>(D);
         pr.p.d_ld = ld_d;

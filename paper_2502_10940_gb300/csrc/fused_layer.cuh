@@ -100,15 +100,10 @@ struct FusedCfg {
     static constexpr int OUT_COL0 = 128;
 };
 
-// UMMA shared-memory descriptor of k-step ks (16 k) of a stage operand:
-// K-major, +32 bytes inside the swizzled 128-byte row; MN-major (64 x 64
-// boxes, one per 64 MN indices, 8 KB apart), +16 rows of 128 bytes.
+// The low descriptor word's step from one k-step (16 k) to the next: K-major,
+// +32 bytes inside the swizzled 128-byte row; MN-major, +16 rows of 128 bytes.
 template <bool MN>
-__device__ __forceinline__ uint64_t fused_operand_desc(uint32_t base, int ks)
-{
-    return MN ? smem_desc_sw128(base + ks * UMMA_K * 128, 64 * BK * 2, 1024)
-              : smem_desc_sw128(base + ks * UMMA_K * 2, 16, 1024);
-}
+constexpr uint32_t FUSED_KSTEP = (MN ? UMMA_K * 128 : UMMA_K * 2) >> 4;
 
 template <int R, bool BWD, int SIG>
 __global__ void __launch_bounds__(NUM_THREADS, 1) fused_layer_kernel(const __grid_constant__ FusedParams P)
@@ -297,7 +292,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) fused_layer_kernel(const __gri
         if (lane == 0) {
             constexpr uint32_t idesc_1 = idesc_bf16_f32(BM, R, 0, BWD ? 1 : 0);
             constexpr uint32_t idesc_2 = idesc_bf16_f32(BM, FBN, 0, BWD ? 1 : 0);
-            const uint32_t t_addr = smem_u32(tbuf);
+            // the low words' address fields step with the stage and the k-step
+            const DescWords desc_in = operand_desc<false>(smem_u32(ring)), desc_w1 = operand_desc<BWD>(smem_u32(ring) + C::IN_BYTES),
+                            desc_w2 = operand_desc<BWD>(smem_u32(ring)), desc_t = operand_desc<false>(smem_u32(tbuf));
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true, issued_any = false;
@@ -322,11 +319,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) fused_layer_kernel(const __gri
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sx = smem_u32(ring + stage * C::STAGE_BYTES);
+                    const uint32_t off = static_cast<uint32_t>(stage * (C::STAGE_BYTES >> 4));
 #pragma unroll
                     for (int ks = 0; ks < BK / UMMA_K; ++ks)
-                        umma_f16(tmem_base, fused_operand_desc<false>(sx, ks),
-                                 fused_operand_desc<BWD>(sx + C::IN_BYTES, ks), idesc_1, (kb > 0 || ks > 0) ? 1u : 0u);
+                        umma_f16(tmem_base, desc_at(desc_in.lo + off + ks * FUSED_KSTEP<false>, desc_in.hi),
+                                 desc_at(desc_w1.lo + off + ks * FUSED_KSTEP<BWD>, desc_w1.hi), idesc_1,
+                                 (kb > 0 || ks > 0) ? 1u : 0u);
                     issued_any = true;
                     umma_commit(&empty_bar[stage]);
                     next();
@@ -351,11 +349,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) fused_layer_kernel(const __gri
                             break;
                         }
                         tc_fence_after();
-                        const uint32_t sb = smem_u32(ring + stage * C::STAGE_BYTES);
-                        const uint32_t sh = t_addr + k2 * (BM * BK * 2);
+                        const uint32_t off = static_cast<uint32_t>(stage * (C::STAGE_BYTES >> 4));
+                        const uint32_t toff = static_cast<uint32_t>(k2 * ((BM * BK * 2) >> 4));
 #pragma unroll
                         for (int ks = 0; ks < BK / UMMA_K; ++ks)
-                            umma_f16(d_y, fused_operand_desc<false>(sh, ks), fused_operand_desc<BWD>(sb, ks), idesc_2,
+                            umma_f16(d_y, desc_at(desc_t.lo + toff + ks * FUSED_KSTEP<false>, desc_t.hi),
+                                     desc_at(desc_w2.lo + off + ks * FUSED_KSTEP<BWD>, desc_w2.hi), idesc_2,
                                      (k2 > 0 || ks > 0) ? 1u : 0u);
                         umma_commit(&empty_bar[stage]);
                         next();

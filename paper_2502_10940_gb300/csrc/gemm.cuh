@@ -32,7 +32,8 @@
 //
 // Epilogues (the elementwise parts of the layer, fused so that the rank-r
 // intermediate makes no extra HBM round trip):
-//   EPI_STORE   D = bf16(acc)                                  (Y, dX)
+//   EPI_STORE   D = bf16(acc)                                  (Y, dX); EPI_STORE64
+//               the same through 64-column boxes, as EPI_STORE on CTA pairs
 //   EPI_ZH      Z = bf16(acc), H = bf16(sigma(Z))              (forward A-GEMM)
 //   EPI_DSIGMA  dZ = bf16(acc * sigma'(Z_saved)); EPI_DSIGMA_H (CoLA-M) also
 //               H = bf16(sigma(Z_saved)) for the weight gradient of B
@@ -95,7 +96,7 @@ enum : unsigned int {
 
 enum Epi : int {
     EPI_STORE = 0, EPI_ZH = 1, EPI_DSIGMA = 2, EPI_F32 = 3, EPI_TAIL = 4, EPI_GLU = 5, EPI_GLU_BWD = 6,
-    EPI_DSIGMA_H = 7, EPI_GLU_BWD_LONG = 8
+    EPI_DSIGMA_H = 7, EPI_GLU_BWD_LONG = 8, EPI_STORE64 = 9
 };
 enum Sigma : int { SIG_IDENTITY = 0, SIG_SILU = 1, SIG_GELU = 2 };
 
@@ -142,8 +143,7 @@ struct GemmParams {
 // one is processed, and dZ is computed in place and TMA-stored from the box.
 constexpr int EPI_BOX_BYTES = 32 * 32 * 2;
 constexpr int EPI_OUT_BOXES = 2;
-static_assert(EPI_OUT_BOXES == 2, "the CTA-pair store epilogue stages a chunk pair into the whole ring");
-constexpr int EPI_WARP_BYTES = EPI_OUT_BOXES * EPI_BOX_BYTES;
+constexpr int EPI_WARP_BYTES = EPI_OUT_BOXES * EPI_BOX_BYTES;   // or one 64-column box
 constexpr int EPI_SMEM_BYTES = NUM_EPI_WARPS * EPI_WARP_BYTES;
 // The gated dX epilogue works on chunks of 64 columns: a box of 32 rows
 // (128-byte rows, 128-byte swizzle) of Y_up and one of Y_gate, TMA-loaded
@@ -642,6 +642,25 @@ __device__ __forceinline__ void store_row8(__nv_bfloat16* d, const uint4& w, int
         if (e < valid) d16[e] = static_cast<uint16_t>((e & 1) ? (v[e >> 1] >> 16) : (v[e >> 1] & 0xFFFFu));
 }
 
+// The UMMA descriptor of an operand tile at shared-memory address `saddr`
+// (K-major, or MN-major as 64 x 64 boxes 8 KB apart), as two words: every k-step
+// and stage of the ring changes only the address field in the low one, so the
+// issuing thread spends one addition on a descriptor.  Forming each descriptor
+// from its fields made the issue the bottleneck of the short MMAs (dX of a
+// 65536 x 512 output, K = 128: 23 us).
+struct DescWords {
+    uint32_t lo, hi;
+};
+
+template <bool MN>
+__device__ __forceinline__ DescWords operand_desc(uint32_t saddr)
+{
+    const uint64_t d = MN ? smem_desc_sw128(saddr, 64 * BK * 2, 1024) : smem_desc_sw128(saddr, 16, 1024);
+    return {static_cast<uint32_t>(d), static_cast<uint32_t>(d >> 32)};
+}
+
+__device__ __forceinline__ uint64_t desc_at(uint32_t lo, uint32_t hi) { return (static_cast<uint64_t>(hi) << 32) | lo; }
+
 // ------------------------------------------------------------ the kernel
 template <int BN, int MSUB, bool A_MN, bool B_MN, int EPI, bool PAIR = false, int SIG = SIG_IDENTITY>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
@@ -670,7 +689,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     constexpr bool GLU_ONE = EPI == EPI_GLU_BWD_LONG;   // one box per slot
     constexpr int WARP_BYTES = epi_warp_bytes(EPI);
     constexpr int ZSLOTS = epi_slots(EPI);          // side-input slots per epilogue warp
-    constexpr int CHUNK = GLU_BWD || EPI == EPI_GLU ? GLU_COLS : 32;   // columns of one epilogue chunk
+    // columns of one epilogue chunk
+    constexpr bool STORE64 = EPI == EPI_STORE64 || (EPI == EPI_STORE && PAIR);
+    constexpr int CHUNK = GLU_BWD || EPI == EPI_GLU || STORE64 ? GLU_COLS : 32;
     constexpr int STAGES = C::STAGES;
     constexpr int TILE_M = C::TILE_M;
     extern __shared__ uint8_t smem_raw[];
@@ -922,6 +943,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         // ------------------------------------------------ MMA issuer
         if (lane == 0 && leader) {   // a pair's MMAs are issued by its even CTA alone
             constexpr uint32_t idesc = idesc_bf16_f32(PAIR ? 2 * BM : BM, BN, A_MN ? 1 : 0, B_MN ? 1 : 0);
+            const DescWords desc_a = operand_desc<A_MN>(smem_u32(smem_a)), desc_b = operand_desc<B_MN>(smem_u32(smem_b));
             int stage = 0;
             uint32_t phase = 0;
             int buf = 0;
@@ -955,20 +977,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(smem_a + stage * C::A_BYTES);
-                    const uint32_t sb = smem_u32(smem_b + stage * C::B_BYTES);
+                    // the stage's descriptors: only their address fields differ
+                    const uint32_t a_lo = desc_a.lo + static_cast<uint32_t>(stage * (C::A_BYTES >> 4));
+                    const uint32_t b_lo = desc_b.lo + static_cast<uint32_t>(stage * (C::B_BYTES >> 4));
 #pragma unroll
                     for (int ks = 0; ks < BK / UMMA_K; ++ks) {
                         // K-major: next 16 k = +32 bytes inside the swizzled 128-byte row.
                         // MN-major: next 16 k = +16 rows of 128 bytes.
-                        const uint64_t db = B_MN ? smem_desc_sw128(sb + ks * UMMA_K * 128, 64 * BK * 2, 1024)
-                                                 : smem_desc_sw128(sb + ks * UMMA_K * 2, 16, 1024);
+                        const uint64_t db = desc_at(b_lo + ks * ((B_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4), desc_b.hi);
 #pragma unroll
                         for (int sub = 0; sub < MSUB; ++sub) {
                             // sub-tile `sub` = A rows [128 sub, 128 sub + 128): +16 KB either way
-                            const uint32_t sas = sa + sub * BM * BK * 2;
-                            const uint64_t da = A_MN ? smem_desc_sw128(sas + ks * UMMA_K * 128, 64 * BK * 2, 1024)
-                                                     : smem_desc_sw128(sas + ks * UMMA_K * 2, 16, 1024);
+                            const uint64_t da = desc_at(a_lo + ks * ((A_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4) +
+                                                            sub * ((BM * BK * 2) >> 4), desc_a.hi);
                             const bool second = EPI == EPI_GLU && kb >= half;
                             const uint32_t acc = (ks > 0 || (kb > kb0 && kb != half)) ? 1u : 0u;
                             const uint32_t d_acc = d_tmem + (second ? BN : 0);
@@ -1244,60 +1265,72 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 }
                 continue;
             }
-            if constexpr (EARLY_FREE) {
-                // EPI_STORE, one 128-row sub-tile: this warp's chunks into
-                // registers as bf16, the accumulator freed at once, then the
-                // stores; the MMAs of the tile after next need not wait for the
-                // stores of this one to drain through the box ring
-                uint32_t wsave[BN / 64][16];
+            if constexpr (STORE64) {
+                // chunks of 64 columns through one box per warp, staged again when
+                // its store has read it (measured against two 32-column boxes behind
+                // one fence, on pairs: Y and dX of 65536 x 2048, K = 512 94.6 -> 92.5
+                // us, dX of 65536 x 5461, whose rows are not 32-byte aligned, 314 ->
+                // 283 us)
+                auto take = [&](int c, uint32_t (&w)[32]) {
 #pragma unroll
-                for (int i = 0; i < BN / 64; ++i) {
-                    const int c = c_first + C_STEP * i;
-                    if (c < nch) {
+                    for (int h = 0; h < 2; ++h) {
                         uint32_t v[32];
-                        tmem_ld_32x32b_x32(tbase + c * 32, v);
+                        tmem_ld_32x32b_x32(tbase + c * GLU_COLS + 32 * h, v);
                         tmem_ld_wait();
 #pragma unroll
                         for (int j = 0; j < 16; ++j)
-                            wsave[i][j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+                            w[16 * h + j] = pack_bf16x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
                     }
+                };
+                auto store = [&](int c, const uint32_t (&w)[32]) {
+                    const int col0 = n_blk * BN + c * GLU_COLS, valid = p.N - col0;
+                    if ((p.N & 7) != 0 && valid < GLU_COLS) {
+                        // a TMA store would write the row padding past a ragged right edge
+                        if (row < p.M) {
+#pragma unroll
+                            for (int j = 0; j < GLU_COLS / 8; ++j)
+                                store_row8(p.d_ptr + row * p.d_ld + col0 + 8 * j,
+                                           make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]), valid - 8 * j);
+                        }
+                    } else {
+                        if (lane == 0) bulk_wait_group_read<0>();
+                        __syncwarp();
+                        stage_row128(ep, lane, [&](int j) { return w[j]; });
+                        fence_proxy_async_smem();
+                        store_box(map_d, ep, col0, row0);
+                    }
+                };
+                auto free_acc = [&]() {
+                    tc_fence_before();
+                    if (PAIR)
+                        mbar_arrive_cluster(mapa_shared(smem_u32(&tempty_bar[buf]), 0));
+                    else
+                        mbar_arrive(&tempty_bar[buf]);
+                };
+                if constexpr (EARLY_FREE) {
+                    // this warp's chunks into registers, the accumulator freed at once:
+                    // the MMAs of the tile after next need not wait for the stores
+                    constexpr int NC = BN / (C_STEP * GLU_COLS);
+                    uint32_t w[NC][32];
+#pragma unroll
+                    for (int i = 0; i < NC; ++i)
+                        if (c_first + C_STEP * i < nch) take(c_first + C_STEP * i, w[i]);
+                    free_acc();
+#pragma unroll
+                    for (int i = 0; i < NC; ++i)
+                        if (c_first + C_STEP * i < nch) store(c_first + C_STEP * i, w[i]);
+                } else {
+#pragma unroll 1
+                    for (int c = c_first; c < nch; c += C_STEP) {
+                        uint32_t w[32];
+                        take(c, w);
+                        store(c, w);
+                    }
+                    free_acc();
                 }
-                tc_fence_before();
-                if (PAIR)
-                    mbar_arrive_cluster(mapa_shared(smem_u32(&tempty_bar[buf]), 0));
-                else
-                    mbar_arrive(&tempty_bar[buf]);
                 if (++buf == 2) {
                     buf = 0;
                     bphase ^= 1u;
-                }
-#pragma unroll
-                for (int i = 0; i < BN / 64; i += 2) {
-                    const int c0 = c_first + C_STEP * i, c1 = c0 + C_STEP;
-                    const bool full = c1 < nch && !((p.N & 7) != 0 && n_blk * BN + c1 * 32 + 32 > p.N) && row0 < cur_M;
-                    if (full) {
-                        // both boxes of the ring at once, behind one proxy fence
-                        // (measured: the 1B Y GEMMs 3 %, the dX GEMMs 2 % faster
-                        // than a fence per box)
-                        if (lane == 0) bulk_wait_group_read<0>();
-                        __syncwarp();
-                        stage_row(ep, lane, wsave[i]);
-                        stage_row(ep + EPI_BOX_BYTES, lane, wsave[i + 1]);
-                        fence_proxy_async_smem();
-                        __syncwarp();
-                        if (lane == 0) {
-                            tma_store_2d(map_d, ep, n_blk * BN + c0 * 32, row0);
-                            tma_store_2d(map_d, ep + EPI_BOX_BYTES, n_blk * BN + c1 * 32, row0);
-                            bulk_commit_group();
-                        }
-                        out_slot = 0;
-                    } else if (c0 < nch) {
-                        // emit waits for all but the newest group, but the newest
-                        // one may be a pair that still reads both boxes
-                        if (lane == 0) bulk_wait_group_read<0>();
-                        put(p, map_d, p.d_ptr, wsave[i], n_blk * BN + c0 * 32, row0, row);
-                        if (c1 < nch) put(p, map_d, p.d_ptr, wsave[i + 1], n_blk * BN + c1 * 32, row0, row);
-                    }
                 }
                 continue;
             }

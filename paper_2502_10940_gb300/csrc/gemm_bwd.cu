@@ -55,7 +55,10 @@ template cudaError_t launch_gemm<256, 1, false, true, EPI_DSIGMA_H, true, SIG_SI
 template cudaError_t launch_gemm<256, 1, false, true, EPI_DSIGMA_H, true, SIG_GELU>(
     const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<128, 1, false, true, EPI_STORE>(const GemmBatch&, int, bool, cudaStream_t);
+template cudaError_t launch_gemm<128, 1, false, true, EPI_STORE64>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<256, 1, false, true, EPI_STORE>(const GemmBatch&, int, bool, cudaStream_t);
+template cudaError_t launch_gemm<256, 1, false, true, EPI_STORE64>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<128, 2, false, true, EPI_STORE>(const GemmBatch&, int, bool, cudaStream_t);
+template cudaError_t launch_gemm<128, 2, false, true, EPI_STORE64>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<256, 1, false, true, EPI_STORE, true>(const GemmBatch&, int, bool, cudaStream_t);
 }  // namespace cola

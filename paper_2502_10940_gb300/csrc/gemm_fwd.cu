@@ -30,8 +30,11 @@ template cudaError_t launch_gemm<256, 1, false, false, EPI_ZH, true, SIG_SILU>(
 template cudaError_t launch_gemm<256, 1, false, false, EPI_ZH, true, SIG_GELU>(
     const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<128, 1, false, false, EPI_STORE>(const GemmBatch&, int, bool, cudaStream_t);
+template cudaError_t launch_gemm<128, 1, false, false, EPI_STORE64>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<256, 1, false, false, EPI_STORE>(const GemmBatch&, int, bool, cudaStream_t);
+template cudaError_t launch_gemm<256, 1, false, false, EPI_STORE64>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<128, 2, false, false, EPI_STORE>(const GemmBatch&, int, bool, cudaStream_t);
+template cudaError_t launch_gemm<128, 2, false, false, EPI_STORE64>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<256, 1, false, false, EPI_STORE, true>(const GemmBatch&, int, bool, cudaStream_t);
 
 // sigma of 8 bf16 values (one 16-byte vector), with the logistic's form L

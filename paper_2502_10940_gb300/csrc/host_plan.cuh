@@ -126,6 +126,19 @@ int fill_bn(int64_t M, int64_t N, int64_t K, int count, int sms)
     return count * ((M + BM - 1) / BM) * ((N + 127) / 128) <= sms ? 128 : 256;
 }
 
+// Whether plain outputs of pitch `ld` (`bytes` of them in the launch) are stored
+// through 64-column boxes (EPI_STORE64, and EPI_STORE on CTA pairs) or through
+// rings of 32-column ones.  64 columns where rows are not 128-byte aligned (a
+// 64-byte row piece then touches a sector more, twice as often): Y of 110691 x
+// 1463, two of them, 297 -> 222 us; and for outputs that L2 takes: Y of 65536 x
+// 512 20.8 -> 19 us.  Larger aligned outputs are bound by HBM writes, which the
+// ring keeps more of in flight: three of 131072 x 1024 199 us with 64 columns,
+// 194 with 32.
+bool store_boxes64(bool pair, int64_t ld, int64_t bytes)
+{
+    return pair || ld % 64 != 0 || bytes <= (96ll << 20);
+}
+
 // Tile modes ("msub" below): 1 = one CTA runs a 128-row tile; 2 = one CTA
 // runs two 128-row sub-tiles sharing each B tile; TILE_PAIR = a CTA pair runs
 // a 256-row tile with tcgen05 cta_group::2 (each CTA loads half of B).
@@ -454,7 +467,7 @@ cudaError_t dispatch_sig(int bn, int msub, GemmBatch& b, int sms, cudaStream_t s
     // 128 x 128 tiles (its long-K form on pairs only)
     constexpr bool small_only = EPI == EPI_F32 && !A_MN;
     constexpr bool glu_bwd = epi_glu_bwd(EPI);
-    if constexpr (!small_only) {
+    if constexpr (!small_only && EPI != EPI_STORE64) {
         if (msub == TILE_PAIR && bn == 256) {
             const int pairs = units < sms / 2 ? units : sms / 2;
             return launch_gemm<256, 1, A_MN, B_MN, EPI, true, SIG>(b, 2 * pairs, pdl, s);

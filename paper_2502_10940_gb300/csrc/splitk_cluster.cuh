@@ -298,6 +298,7 @@ __global__ void __launch_bounds__(CRED_THREADS, 1) splitk_cluster_kernel(const _
         // ------------------------------------------------ MMA issuer
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_bf16_f32(BM, CBN, A_MN ? 1 : 0, B_MN ? 1 : 0);
+            const DescWords desc_a = operand_desc<A_MN>(smem_u32(smem_a)), desc_b = operand_desc<B_MN>(smem_u32(smem_b));
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true, issued_any = false;
@@ -307,16 +308,14 @@ __global__ void __launch_bounds__(CRED_THREADS, 1) splitk_cluster_kernel(const _
                     break;
                 }
                 tc_fence_after();
-                const uint32_t sa = smem_u32(smem_a + stage * C::A_BYTES);
-                const uint32_t sb = smem_u32(smem_b + stage * C::B_BYTES);
+                const uint32_t a_lo = desc_a.lo + static_cast<uint32_t>(stage * (C::A_BYTES >> 4));
+                const uint32_t b_lo = desc_b.lo + static_cast<uint32_t>(stage * (C::B_BYTES >> 4));
 #pragma unroll
                 for (int ks = 0; ks < BK / UMMA_K; ++ks) {
-                    // next 16 k: +16 rows of 128 bytes (MN-major, 64-column groups 8 KB
-                    // apart) or +32 bytes inside the swizzled row (K-major)
-                    const uint64_t da = A_MN ? smem_desc_sw128(sa + ks * UMMA_K * 128, 64 * BK * 2, 1024)
-                                             : smem_desc_sw128(sa + ks * UMMA_K * 2, 16, 1024);
-                    const uint64_t db = B_MN ? smem_desc_sw128(sb + ks * UMMA_K * 128, 64 * BK * 2, 1024)
-                                             : smem_desc_sw128(sb + ks * UMMA_K * 2, 16, 1024);
+                    // next 16 k: +16 rows of 128 bytes (MN-major) or +32 bytes inside the
+                    // swizzled row (K-major)
+                    const uint64_t da = desc_at(a_lo + ks * ((A_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4), desc_a.hi);
+                    const uint64_t db = desc_at(b_lo + ks * ((B_MN ? UMMA_K * 128 : UMMA_K * 2) >> 4), desc_b.hi);
                     umma_f16(tmem_base, da, db, idesc, (kb > kb0 || ks > 0) ? 1u : 0u);
                 }
                 issued_any = true;

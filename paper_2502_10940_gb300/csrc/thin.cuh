@@ -271,6 +271,7 @@ __global__ void __launch_bounds__(THIN_THREADS) thin_kernel(const __grid_constan
         // ------------------------------------------------ MMA issuer
         if (lane == 0) {
             const uint32_t idesc = idesc_bf16_f32(BM, NT, 0, 0);
+            const DescWords desc_w = operand_desc<false>(smem_u32(smem)), desc_t = operand_desc<false>(smem_u32(smem) + BM * BK * 2);
             bool ok = true, issued_any = false;
             for (int i = 0; i < iters; ++i) {
                 const int s = i % stages;
@@ -279,13 +280,13 @@ __global__ void __launch_bounds__(THIN_THREADS) thin_kernel(const __grid_constan
                     break;
                 }
                 tc_fence_after();
-                const uint32_t sw = smem_u32(smem + s * stage_bytes);
-                const uint32_t st = sw + BM * BK * 2;
+                const uint32_t off = (s * stage_bytes) >> 4;
                 const uint32_t acc = tmem_base + static_cast<uint32_t>(GLU && (i & 1) ? NT : 0);
 #pragma unroll
                 for (int ks = 0; ks < BK / UMMA_K; ++ks)
-                    umma_f16(acc, smem_desc_sw128(sw + ks * UMMA_K * 2, 16, 1024),
-                             smem_desc_sw128(st + ks * UMMA_K * 2, 16, 1024), idesc, (i >= HALVES || ks > 0) ? 1u : 0u);
+                    umma_f16(acc, desc_at(desc_w.lo + off + ks * (UMMA_K * 2 >> 4), desc_w.hi),
+                             desc_at(desc_t.lo + off + ks * (UMMA_K * 2 >> 4), desc_t.hi), idesc,
+                             (i >= HALVES || ks > 0) ? 1u : 0u);
                 issued_any = true;
                 umma_commit(&empty_bar[s]);
             }
