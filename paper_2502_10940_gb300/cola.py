@@ -151,6 +151,11 @@ def _ptr(t):
 
 def _stream(s):
     if s is None:
+        # the raw handle of the current device's current stream, without the
+        # Stream object torch.cuda.current_stream() builds around it (3 us of
+        # the 8 to 14 us a small forward call takes on the host)
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(s, int):
         return s
