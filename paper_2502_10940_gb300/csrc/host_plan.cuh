@@ -81,29 +81,41 @@ bool map_mnmajor(CUtensorMap* m, const void* base, int64_t mn_extent, int64_t k_
 }
 
 // ------------------------------------------------------------ planning
-// Column tile: the width that pads N least; a compute-heavy GEMM (see
-// heavy_gemm) takes 256 whenever that pads N by at most 5 %, because only
-// 256-column tiles run on CTA pairs.
-int choose_bn(int64_t N, bool heavy = false)
+// Column tile: the width that pads N least; a compute-heavy GEMM with K >= 512
+// (`pairs`) takes 256, because only 256-column tiles run on CTA pairs, which
+// outweighs the padding (at most a third of the tile columns).  Measured against
+// 128-column tiles wherever 256 pads N by more than 5 % (forward + backward):
+// 16384 tokens 2600 -> 2600, r = 640 396 -> 301 us; 12000, 3300 -> 3300, r = 832
+// 427 -> 357; 65536, 1500 -> 1500, r = 384 479 -> 439.
+int choose_bn(int64_t N, bool pairs = false)
 {
     if (N <= 128) return 128;
+    if (pairs) return 256;
     const int64_t pad256 = (N + 255) / 256 * 256;
     const int64_t pad128 = (N + 127) / 128 * 128;
-    if (heavy && N >= 1024 && pad256 * 100 <= N * 105) return 256;
     return pad256 <= pad128 ? 256 : 128;
 }
 
-// Compute-heavy: more than one 128-row block and either >= 64 GFLOP, or
-// >= 16 GFLOP at an arithmetic intensity (each operand read once, the
-// result written once) of >= 300 FLOP/B, above the ridge of the GB300 bf16
-// roofline (~287).  The second clause takes the tensor-bound GEMMs of the
-// 8192-token inference workloads (measured: 1B forward -14 %).
+// Compute-heavy: more than one 128-row block and
+//   - at least 64 GFLOP, or
+//   - at least 16 GFLOP at an arithmetic intensity (each operand read once, the
+//     result written once) of >= 300 FLOP/B, above the ridge of the GB300 bf16
+//     roofline (~287): the tensor-bound GEMMs of the 8192-token inference
+//     workloads (measured: 1B forward -14 %), or
+//   - at least 16 GFLOP at >= 150 FLOP/B with K >= 1024, where the walk is long
+//     against the epilogue, and with K >= 2048 if 256-column tiles pad N more
+//     (forward + backward: 32768 tokens 1024 -> 2736, r = 256 243 -> 227 us,
+//     100000, 1000 -> 1100, r = 192 407 -> 373; but 30000, 1200 -> 1200, r = 320
+//     without the second condition 215 -> 226, and the 65536-token q/k/v of the
+//     60M block, K = 512, 41 -> 48 us for Z).
 bool heavy_gemm(int64_t M, int64_t N, int64_t K)
 {
     const double m = static_cast<double>(M), n = static_cast<double>(N), k = static_cast<double>(K);
     const double flops = 2.0 * m * n * k;
-    const double bytes = 2.0 * (m * k + n * k + m * n);
-    return M > 128 && (flops >= 64e9 || (flops >= 16e9 && flops / bytes >= 300.0));
+    const double intensity = flops / (2.0 * (m * k + n * k + m * n));
+    if (M <= 128 || flops < 16e9) return false;
+    const bool pads = (N + 255) / 256 * 256 > (N + 127) / 128 * 128;
+    return flops >= 64e9 || intensity >= 300.0 || (intensity >= 150.0 && K >= (pads ? 2048 : 1024));
 }
 
 // A GEMM of one 128-row block (a few tokens: decode) streams its B operand
@@ -114,7 +126,7 @@ bool heavy_gemm(int64_t M, int64_t N, int64_t K)
 int choose_bn_for(int64_t M, int64_t N, int64_t K)
 {
     if (M <= 128 && N <= 8192) return 128;
-    return choose_bn(N, heavy_gemm(M, N, K));
+    return choose_bn(N, heavy_gemm(M, N, K) && K >= 512);
 }
 
 // The same for `count` GEMMs of one launch, with 128 columns where those tiles
