@@ -364,12 +364,14 @@ cola_status_t run_cluster_wgrad(int count, const CredJob* jobs, int64_t ntok, in
 }
 
 // The cluster split of a weight-gradient group (128 x 128 tiles, at most 8
-// splits, one wave of clusters): > 1 when it applies -- each CTA walks at
-// most CLUSTER_MAX_KPS k-blocks -- and its k-blocks per CTA undercut the
-// planned schedule with its reduce launch.  Its 4-stage, one-tile-per-CTA
-// form is made for short token walks: at 65536 tokens (the LLaMA-60M block,
-// 128-171 k-blocks per CTA) it ran the weight gradients 60 -> 93 us.
+// splits): > 1 when it applies -- each CTA walks at most CLUSTER_MAX_KPS
+// k-blocks -- and its k-block steps undercut the planned schedule with its
+// reduce launch.  Its 4-stage, one-tile-per-CTA form is made for short token
+// walks: at 65536 tokens (the LLaMA-60M block, 128-171 k-blocks per CTA) it ran
+// the weight gradients 60 -> 93 us.  Walks so short that the most splits leave a
+// CTA at most CLUSTER_SHORT_KPS k-blocks take those, also in two waves.
 constexpr int CLUSTER_MAX_KPS = 32;
+constexpr int CLUSTER_SHORT_KPS = 8;
 
 int wgrad_cluster_splits(const WgradPlan& w, int64_t ntok, int accumulate_f32, int sms)
 {
@@ -378,14 +380,20 @@ int wgrad_cluster_splits(const WgradPlan& w, int64_t ntok, int accumulate_f32, i
     for (int j = 0; j < w.count; ++j)
         tiles += static_cast<int>(((w.p[j].M + BM - 1) / BM) * ((w.p[j].N + CBN - 1) / CBN));
     const int kb = static_cast<int>((ntok + BK - 1) / BK);
-    const int S = cluster_splits(tiles, kb, sms);
+    if (tiles < 1 || 2 * tiles > sms) return 1;
+    int cost = 0;
+    int S = std::min(std::min(sms / tiles, MAX_CLUSTER), kb / 4);
+    if (S >= 2 && (kb + S - 1) / S <= CLUSTER_SHORT_KPS)
+        cost = (kb + S - 1) / S;
+    else
+        S = cluster_splits(tiles, kb, sms, &cost);
     if (S < 2 || (kb + S - 1) / S > CLUSTER_MAX_KPS) return 1;
     double planned = w.cost;
     if (!accumulate_f32) {
         const TailPlan tp = wgrad_tail_plan(w, ntok, sms);
         if (tail_wins(w, tp)) planned = tp.cost;
     }
-    return (kb + S - 1) / S <= planned ? S : 1;
+    return cost <= planned ? S : 1;
 }
 
 // One rank-r GEMM of few output tiles, D_j [n x N] for j < count over K, its K

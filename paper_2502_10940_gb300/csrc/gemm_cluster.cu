@@ -2,6 +2,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <mutex>
 
 #define COLA_DEFINE_CLUSTER_KERNEL
 #include "splitk_cluster.cuh"
@@ -43,6 +44,40 @@ cudaError_t launch_one(const CredBatch& b, bool pdl, cudaStream_t stream)
 }
 
 }  // namespace
+
+// Clusters of S CTAs that the current device runs at once, asked once per device.
+const int* reduce_cluster_capacity(int sms)
+{
+    struct Caps {
+        std::once_flag once;
+        int n[MAX_CLUSTER + 1];
+    };
+    static Caps caps[65];   // [64]: no device, or one beyond the table
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 64;
+    Caps& c = caps[dev];
+    std::call_once(c.once, [&] {
+        const auto kern = splitk_cluster_kernel<true, true, CRED_STORE, SIG_IDENTITY>;
+        const bool set = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, CredCfg::SMEM_BYTES) == cudaSuccess;
+        for (int s = 0; s <= MAX_CLUSTER; ++s) {
+            c.n[s] = s > 0 && sms >= s ? sms / s : 1;
+            if (s < 2 || !set) continue;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(static_cast<unsigned>(s));
+            cfg.blockDim = dim3(CRED_THREADS);
+            cfg.dynamicSmemBytes = CredCfg::SMEM_BYTES;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = static_cast<unsigned>(s);
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0) c.n[s] = n;
+        }
+    });
+    return c.n;
+}
 
 cudaError_t launch_splitk_cluster(const CredBatch& b, int op, int sigma, bool pdl, cudaStream_t stream)
 {

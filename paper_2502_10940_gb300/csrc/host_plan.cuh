@@ -14,6 +14,11 @@
 #include "thin.cuh"
 
 namespace cola {
+
+// Thread-block clusters of S CTAs (index S, at least 1) of the cluster-reduced
+// kernel that the current device runs at once.
+const int* reduce_cluster_capacity(int sms);
+
 namespace {
 
 // ------------------------------------------------------------ tensor maps
@@ -245,16 +250,32 @@ int small_launch_splits(int tiles, int k_blocks, int sms)
 }
 
 // K splits of a small launch reduced inside thread-block clusters
-// (splitk_cluster.cuh, 128 x 128 tiles): with fewer tiles than half the SMs,
-// the largest S <= 8 that keeps tiles * S within the SMs and >= 4 k-blocks
-// per split.  1 = no split.
-int cluster_splits(int tiles, int k_blocks, int sms)
+// (splitk_cluster.cuh, 128 x 128 tiles), with at most half as many tiles as SMs,
+// up to S = 8 and >= 4 k-blocks per split.  The SMs of a cluster lie in one
+// partition of the GPU, so it runs fewer clusters of S at once than SMs / S (on
+// GB300 76, 46, 36, 28, 23, 15, 15 for S = 2..8): S is the one whose waves of
+// clusters take the fewest k-block steps, CLUSTER_WAVE_KB of them for the
+// exchange and the start of each wave.  Measured (weight gradients of 15249
+// tokens, 19 tiles): S = 8 in two waves 36 us, planned split and reduce 28.
+// *cost (when not null): those steps, less one wave's CLUSTER_WAVE_KB.
+// 1 = no split.
+constexpr int CLUSTER_WAVE_KB = 8;
+
+int cluster_splits(int tiles, int k_blocks, int sms, int* cost = nullptr)
 {
     if (tiles < 1 || 2 * tiles > sms) return 1;
-    int s = sms / tiles;
-    if (s > MAX_CLUSTER) s = MAX_CLUSTER;
-    if (s > k_blocks / 4) s = k_blocks / 4;
-    return s < 1 ? 1 : s;
+    const int* cap = reduce_cluster_capacity(sms);
+    int best = 1, best_cost = 0;
+    for (int s = 2; s <= MAX_CLUSTER && s <= k_blocks / 4 && s * tiles <= sms; ++s) {
+        const int waves = (tiles + cap[s] - 1) / cap[s];
+        const int c = waves * ((k_blocks + s - 1) / s + CLUSTER_WAVE_KB) - CLUSTER_WAVE_KB;
+        if (best == 1 || c <= best_cost) {
+            best = s;
+            best_cost = c;
+        }
+    }
+    if (cost) *cost = best_cost;
+    return best;
 }
 
 // K splits, inside clusters, of the `count` rank-r GEMMs of one launch (Z of the
@@ -288,8 +309,7 @@ void thin_splits(ThinBatch& b, bool glu, int sms)
     b.kps = (b.k_blocks + s - 1) / s;
     b.S = (b.k_blocks + b.kps - 1) / b.kps;   // no empty split
     b.TB = (b.n + b.S - 1) / b.S;
-    constexpr int budget = 110 * 1024;
-    const int left = budget - 1024 - THIN_BAR_BYTES - thin_recv_bytes(b.S, b.TB, glu);
+    const int left = THIN_SMEM_BUDGET - 1024 - THIN_BAR_BYTES - thin_recv_bytes(b.S, b.TB, glu);
     b.stages = left / thin_stage_bytes(b.NT);
     const int iters = b.kps * (glu ? 2 : 1);
     if (b.stages > iters) b.stages = iters;

@@ -88,6 +88,7 @@ __host__ __device__ constexpr int thin_ring_bytes(int stages, int NT, bool glu)
 }
 __host__ __device__ constexpr int thin_recv_bytes(int S, int TB, bool glu) { return S > 1 ? S * TB * BM * 4 * (glu ? 2 : 1) : 0; }
 constexpr int THIN_BAR_BYTES = 256;
+constexpr int THIN_SMEM_BUDGET = 110 * 1024;   // two CTAs per SM
 __host__ __device__ constexpr int thin_smem_bytes(int stages, int NT, int S, int TB, bool glu)
 {
     return 1024 + thin_ring_bytes(stages, NT, glu) + thin_recv_bytes(S, TB, glu) + THIN_BAR_BYTES;

@@ -36,17 +36,19 @@ def _rel(got, ref):
     return float((got.float() - ref).norm() / ref.norm())
 
 
-# n, d_in, d_out, r, projections, Z splits, dZ splits (0: not in a cluster)
-SHAPES = [(65, 520, 600, 192, 1, 2, 2), (130, 4100, 3000, 64, 2, 8, 8), (300, 1000, 2000, 256, 3, 4, 8), (509, 1024, 1024, 256, 3, 4, 4),
-          (1155, 1728, 1728, 512, 1, 3, 3), (1700, 2050, 2050, 192, 1, 5, 5), (2400, 1500, 1500, 256, 1, 4, 4),
-          (4864, 1100, 1100, 128, 2, 2, 2), (4865, 1100, 1100, 192, 1, 0, 0), (2048, 512, 777, 256, 2, 2, 2)]
+# n, d_in, d_out, r, projections, whether Z and dZ split over K in clusters (how
+# many ways depends on how many clusters the device runs at once)
+SHAPES = [(65, 520, 600, 192, 1, True), (130, 4100, 3000, 64, 2, True), (300, 1000, 2000, 256, 3, True),
+          (509, 1024, 1024, 256, 3, True), (1155, 1728, 1728, 512, 1, True), (1700, 2050, 2050, 192, 1, True),
+          (2400, 1500, 1500, 256, 1, True), (4864, 1100, 1100, 128, 2, True), (4865, 1100, 1100, 192, 1, False),
+          (2048, 512, 777, 256, 2, True)]
 
 
 @pytest.mark.parametrize("shape", SHAPES, ids=str)
 @pytest.mark.parametrize("mode,sigma", [("cola", "silu"), ("cola_m", "gelu"), ("cola_m", "silu"), ("cola", "identity")])
 def test_rank_gemms_in_clusters(shape, mode, sigma):
     from paper_2502_10940_gb300 import cola
-    n, d_in, d_out, r, c, sz, sdz = shape
+    n, d_in, d_out, r, c, clustered = shape
     lx, ly = I.padded_ld(d_in), I.padded_ld(d_out)
     X = I.normal_bf16(n, d_in, 1.0, 1, "cuda", ld=lx)
     A = I.normal_bf16(c * r, d_in, d_in ** -0.5, 2, "cuda", ld=lx)
@@ -68,9 +70,10 @@ def test_rank_gemms_in_clusters(shape, mode, sigma):
             cola.cola_fwd_shared_x(d, X, A, B, Y, Z, H, ws)
             cola.cola_bwd_shared_x(d, X, A, B, dY, Z, H, dX, dA, dB, ws)
     assert cola.cola_check_status(ws) == (0, 0)
-    for kind, want in (("fwd_zh", sz), ("bwd_dz", sdz)):
+    for kind in ("fwd_zh", "bwd_dz"):
         rec = [t for t in tr.records() if t[0] == kind]
-        assert len(rec) == 1 and (rec[0][2] if rec[0][3] & CLUSTER else 0) == want, (kind, tr.records())
+        assert len(rec) == 1 and bool(rec[0][3] & CLUSTER) == clustered, (kind, tr.records())
+        assert (2 <= rec[0][2] <= 8) if clustered else rec[0][2] == 1
     f = torch.Tensor.float
     # one bf16 rounding (1.1e-3 as a whole) for Z and H, two to three chained ones
     # for the others (2.4e-3 to 3.2e-3 measured)
