@@ -120,13 +120,16 @@ cola_status_t cola_workspace_init(void* ws, void* stream);
  *                   NULL under COLA_MODE_INFER (Z is then never stored).
  *   H_save [n x r]: output under COLA_MODE_COLA; must be NULL under COLA_M
  *                   and INFER (H is then formed in the workspace and not kept).
- * Two tensor-core GEMMs: Z/H (sigma fused in the epilogue), then Y.  For
- * r = 64 or 128 when both products are HBM-bound (neither compute-heavy nor
- * split over K) and n is at most 128 tokens per SM (19456 on GB300), one
- * kernel instead: each CTA keeps the H of its 128-row tile in shared memory
- * between the two products (H is an intermediate of Eq. (main-fwd), not an
- * output), storing Z and H only as the mode saves them; the results are the
- * same bit for bit (cola_set_fused_forward). */
+ * Two tensor-core GEMMs: Z/H (sigma fused in the epilogue), then Y.  With few
+ * output tiles their K ranges are split over thread-block clusters that add the
+ * partials on chip (cola_set_cluster_splitk; always with at most 32 tokens, or
+ * 64 at r >= 256).  For r = 64 or 128 when both products are HBM-bound (neither
+ * compute-heavy nor, at d_in >= 1024, of fewer tiles than half the SMs) and n is
+ * at most 128 tokens per SM (19456 on GB300), one kernel instead: each CTA keeps
+ * the H of its 128-row tile in shared memory between the two products (H is an
+ * intermediate of Eq. (main-fwd), not an output), storing Z and H only as the
+ * mode saves them; the results are the same bit for bit
+ * (cola_set_fused_forward). */
 cola_status_t cola_fwd(const cola_desc_t* desc, const void* X, const void* A, const void* B, void* Y,
                        void* Z_save, void* H_save, void* ws, size_t ws_bytes, void* stream);
 
@@ -139,7 +142,8 @@ cola_status_t cola_fwd(const cola_desc_t* desc, const void* X, const void* A, co
  * NULL under COLA_M, where H = sigma(Z_save) is recomputed into the
  * workspace).  Outputs dX (bf16), dA and dB (bf16, or fp32 accumulated when
  * desc->wgrad_fp32).  The result does not depend on the mode, bit for bit.
- * Launches: the dZ GEMM (sigma' fused in its epilogue), the weight-gradient
+ * Launches: the dZ GEMM (sigma' fused in its epilogue; with few tiles its K
+ * range split over clusters, cola_set_cluster_splitk), the weight-gradient
  * GEMMs (and their token-split reduce), the dX GEMM.  For r = 64 or 128 when
  * neither the dZ nor the dX GEMM is compute-heavy and n is at most 128
  * tokens per SM, dZ and dX run as one kernel instead: each CTA keeps the dZ
@@ -360,7 +364,7 @@ typedef enum {
     COLA_KERNEL_FWD_Y = 1,       /* Y = H B^T                             (M=n, N=d_out, K=r) */
     COLA_KERNEL_BWD_DZ = 2,      /* dZ = (dY B) * sigma'(Z)               (M=n, N=r, K=d_out) */
     COLA_KERNEL_WGRAD = 3,       /* dB = dY^T H and dA = dZ^T X, token split (M=d_out | r, N=r | d_in, K=n) */
-    COLA_KERNEL_REDUCE = 4,      /* fixed-order sum of the partials       (M, N of the gradient, K=splits) */
+    COLA_KERNEL_REDUCE = 4,      /* fixed-order sum of the partials       (M, N of the result, K=splits) */
     COLA_KERNEL_BWD_DX = 5,      /* dX = dZ A                             (M=n, N=d_in, K=r or 3r) */
     COLA_KERNEL_SIGMA = 6,       /* H = sigma(Z), elementwise             (M=n, N=count r, K=0) */
     COLA_KERNEL_FWD_GLU = 7,     /* M = (H_gate B_gate^T) * (H_up B_up^T) (M=n, N=d_ff, K=2r) */
@@ -376,7 +380,7 @@ typedef struct {
     int32_t kernel;     /* cola_kernel_t */
     int32_t count;      /* GEMMs (or reductions) this one launch runs, 1..4 */
     int32_t mnk[4][3];  /* M, N, K of each (reductions: M, N, splits) */
-    int32_t splits;     /* token splits (weight gradients), else 1 */
+    int32_t splits;     /* splits of the K range (weight gradients: of the tokens), else 1 */
     int32_t flags;      /* bit 0: the epilogue also wrote H (CoLA forward or CoLA-M backward);
                            bit 1: a forward GEMM split over K into fp32 partials (the reduce
                                   launch after it applies the epilogue);
@@ -408,15 +412,18 @@ cola_status_t cola_set_fused_forward(int32_t enable);
  * the same results bit for bit.  enable outside {0, 1}: COLA_ERR_INVALID. */
 cola_status_t cola_set_fused_backward(int32_t enable);
 
-/* Weight-gradient launches with few output tiles and a short token walk (a
- * few thousand tokens) split their tokens to fill the SMs.  1 (default): the
- * splits of a 128 x 128 gradient tile run as one thread-block cluster of up
- * to 8 CTAs that adds the partial tiles on chip, in a fixed order, and
- * stores (or accumulates) in the same launch; 0: the planned split with fp32
- * partials in the workspace and a reduce launch.  The two add the same
- * partials in the same order only when they split alike, so results may
- * differ in the last bits between the settings (each is deterministic run
- * to run).  enable outside {0, 1}: COLA_ERR_INVALID. */
+/* Launches of few output tiles split their K range to fill the SMs: the weight
+ * gradients with a short token walk (a few thousand tokens), and the rank-r
+ * products Z = X A^T and dZ = dY B of up to a few thousand tokens.  1
+ * (default): the splits of a 128 x 128 tile run as one thread-block cluster of
+ * up to 8 CTAs that adds the partial tiles on chip, in a fixed order, and
+ * applies the epilogue in the same launch; 0: weight gradients and Z/H with
+ * fp32 partials in the workspace and a reduce launch, dZ unsplit.  The two add
+ * the same partials in the same order only when they split alike, so results
+ * may differ in the last bits between the settings (each is deterministic run
+ * to run).  The forward GEMMs of at most 32 tokens (64 at r >= 256) always
+ * reduce in clusters.  How many ways a tile is split depends on how many
+ * clusters the device runs at once.  enable outside {0, 1}: COLA_ERR_INVALID. */
 cola_status_t cola_set_cluster_splitk(int32_t enable);
 
 /* Static description of a status code. */

@@ -158,7 +158,8 @@ TailPlan wgrad_tail_plan(const WgradPlan& w, int64_t ntok, int sms)
 bool tail_wins(const WgradPlan& w, const TailPlan& t) { return t.cost <= w.cost; }
 
 // fp32 partial elements the forward of `nproj` projections needs when its
-// GEMMs are small enough to be split over K (small_launch_splits)
+// GEMMs are small enough to be split over K into slabs (small_launch_splits),
+// whichever way cola_set_cluster_splitk is set
 int64_t fwd_part_elems(const cola_desc_t& d, int nproj, int sms)
 {
     int64_t need = 0;
@@ -196,7 +197,7 @@ WsLayout ws_layout(const cola_desc_t& d, int nproj, int sms)
     L.h_off = off;
     if (d.mode != COLA_MODE_COLA) off += align_up(static_cast<size_t>(d.n) * R * 2);
     L.part_off = off;
-    // fp32 partials: of the split-K forward GEMMs of small launches, or of the
+    // fp32 partials: of the slab-split forward GEMMs of small launches, or of the
     // weight gradients (the forward and backward calls use them in turn)
     size_t part = static_cast<size_t>(fwd_part_elems(d, nproj, sms)) * 4;
     if (d.mode != COLA_MODE_INFER) {
@@ -479,8 +480,9 @@ cola_status_t run_f1(const Shape& s, int sigma, int64_t N, const void* X, const 
     COLA_MAP(map_kmajor(&pr.map_b, A, s.d_in, N, s.ld_a, b_box_rows(bn, ms)));
     const int S = ms == 1 ? small_launch_splits(pr.p.m_tiles * pr.p.n_tiles, pr.p.k_blocks, sms) : 1;
     if (S > 1) {
-        // a small launch: K split across CTAs into fp32 partials, then the
-        // reduce applies the Z/H epilogue (Z = bf16(sum), H = bf16(sigma(Z)))
+        // a small launch with the cluster reduction switched off: K split across
+        // CTAs into fp32 partials, then the reduce applies the Z/H epilogue
+        // (Z = bf16(sum), H = bf16(sigma(Z)))
         set_splits(pr.p, S);
         const int64_t slab = partial_elems(pr.p, bn, 1);
         if (static_cast<size_t>(pr.p.splits * slab) * 4 > part_bytes) return COLA_ERR_WORKSPACE;
@@ -536,8 +538,8 @@ std::atomic<int> g_fused_bwd{1};
 
 // The single-kernel forward applies to one layer with r = 64 or 128 whose
 // two GEMMs are HBM-bound (neither is compute-heavy), with at most one
-// 128-row tile per SM, and not split over K (small launches keep the
-// split-K forward).  Measured at 2048 tokens: -10 to -13 % against the two
+// 128-row tile per SM, and with too short a K to be split
+// (small_launch_splits).  Measured at 2048 tokens: -10 to -13 % against the two
 // GEMMs; at 65536 tokens it was 5-13 % slower, so larger launches keep them.
 bool fused_fwd_form(const Shape& s, int sms)
 {

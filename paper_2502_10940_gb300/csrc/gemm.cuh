@@ -25,10 +25,11 @@
 //               accumulators (double buffered, so the epilogue of tile i
 //               overlaps the main loop of tile i+1); allocates TMEM.
 //   warps 2..9  epilogue, two warps per TMEM lane quarter taking alternate
-//               32-column chunks: tcgen05.ld -> fused elementwise -> 32x32
-//               boxes staged in shared memory (64-byte swizzle, bank-conflict
-//               free) -> TMA bulk tensor stores, which are coalesced,
-//               asynchronous and clipped to the tensor's extents in hardware.
+//               chunks of 32 or 64 columns: tcgen05.ld -> fused elementwise ->
+//               boxes of 32 rows staged in shared memory (64- or 128-byte
+//               swizzle, bank-conflict free) -> TMA bulk tensor stores, which are
+//               coalesced, asynchronous and clipped to the tensor's extents in
+//               hardware.
 //
 // Epilogues (the elementwise parts of the layer, fused so that the rank-r
 // intermediate makes no extra HBM round trip):
@@ -38,8 +39,8 @@
 //   EPI_DSIGMA  dZ = bf16(acc * sigma'(Z_saved)); EPI_DSIGMA_H (CoLA-M) also
 //               H = bf16(sigma(Z_saved)) for the weight gradient of B
 //   EPI_F32     fp32 split-K partial slab, reduced (in a fixed order) by the
-//               reduce kernel: fp32-accumulated weight gradients, and the
-//               forward GEMMs of small launches
+//               reduce kernel: weight gradients split uniformly, and the forward
+//               GEMMs of small launches that no cluster reduces
 //   EPI_GLU     gated MLP forward (Fig. 4): the K walk covers [H_gate H_up]
 //               (2r columns of H_cat); the gate half accumulates H_gate B_gate^T
 //               and the up half H_up B_up^T into a second accumulator of the
@@ -137,10 +138,13 @@ struct GemmParams {
 };
 
 // Epilogue staging: per epilogue warp two 2 KB boxes of 32 rows x 32 bf16
-// columns (64-byte rows, 64-byte TMA swizzle).  EPI_STORE / EPI_ZH / EPI_GLU
-// use them as a ring of output boxes.  EPI_DSIGMA uses them as a double buffer for the
-// saved Z: the box of the warp's next chunk is TMA-loaded while the current
-// one is processed, and dZ is computed in place and TMA-stored from the box.
+// columns (64-byte rows, 64-byte TMA swizzle).  EPI_STORE / EPI_ZH / EPI_TAIL
+// use them as a ring of output boxes, EPI_STORE64 and the plain stores of CTA
+// pairs both as one box of 64 columns.  EPI_DSIGMA uses them as a double buffer
+// for the saved Z: the box of the warp's next chunk is TMA-loaded while the
+// current one is processed, and dZ is computed in place and TMA-stored from the
+// box.  (Z, dZ through 64-column boxes as the gated dX epilogue below: K = 1024,
+// r = 256 52 -> 50 us a GEMM, but K >= 1376 2 % and r = 192 4 % slower.)
 constexpr int EPI_BOX_BYTES = 32 * 32 * 2;
 constexpr int EPI_OUT_BOXES = 2;
 constexpr int EPI_WARP_BYTES = EPI_OUT_BOXES * EPI_BOX_BYTES;   // or one 64-column box

@@ -1,7 +1,6 @@
 // Backward activation-gradient GEMMs: dZ = (dY B) * sigma'(Z) (EPI_DSIGMA; with
-// H = sigma(Z) for CoLA-M, EPI_DSIGMA_H) and
-// dX = dZ A (EPI_STORE); A operand K-major, B operand (a weight read
-// transposed) MN-major.
+// H = sigma(Z) for CoLA-M, EPI_DSIGMA_H) and dX = dZ A (EPI_STORE, EPI_STORE64);
+// A operand K-major, B operand (a weight read transposed) MN-major.
 #define COLA_DEFINE_LAUNCHERS
 #include "gemm_launch.cuh"
 

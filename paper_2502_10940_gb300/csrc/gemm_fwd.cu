@@ -1,5 +1,5 @@
-// Forward GEMMs: Z/H = sigma-epilogue of X A^T (EPI_ZH) and Y = H B^T (EPI_STORE);
-// both operands K-major.  Also the elementwise H = sigma(Z) that the CoLA-M
+// Forward GEMMs: Z/H = sigma-epilogue of X A^T (EPI_ZH) and Y = H B^T (EPI_STORE,
+// EPI_STORE64); both operands K-major.  Also the elementwise H = sigma(Z) that the CoLA-M
 // up-projection recompute runs before its Y GEMM.
 #define COLA_DEFINE_LAUNCHERS
 #include "gemm_launch.cuh"

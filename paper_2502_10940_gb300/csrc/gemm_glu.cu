@@ -3,9 +3,10 @@
 // CoLA layers).  Forward (EPI_GLU): Y_gate = H_gate B_gate^T and
 // Y_up = H_up B_up^T of one output tile in two accumulators of one CTA (CTA
 // pair), stored as M = Y_gate * Y_up; both operands K-major: 256 x 256
-// tiles on CTA pairs, 128 x 128 tiles on single CTAs.  Backward (EPI_GLU_BWD): the down layer's dX GEMM, whose epilogue
-// turns dM into dY_gate = dM * Y_up and dY_up = dM * Y_gate; A operand
-// K-major, B operand (the down layer's A factor read transposed) MN-major.
+// tiles on CTA pairs, 128 x 128 tiles on single CTAs.  Backward (EPI_GLU_BWD,
+// EPI_GLU_BWD_LONG): the down layer's dX GEMM, whose epilogue turns dM into
+// dY_gate = dM * Y_up and dY_up = dM * Y_gate; A operand K-major, B operand (the
+// down layer's A factor read transposed) MN-major.
 #define COLA_DEFINE_LAUNCHERS
 #include "gemm_launch.cuh"
 

@@ -5,8 +5,8 @@
 // sums the pieces), or split every tile's token range uniformly into fp32
 // partial slabs that splitk_reduce_kernel sums in a fixed order; fp32
 // gradients accumulated into always take the uniform split.  The same
-// reduce finishes the split-K forward GEMMs of small launches (instantiated
-// here too), applying the Z/H epilogue for the Z GEMM.
+// reduce finishes the forward GEMMs of small launches that are split over K
+// into slabs (instantiated here too), applying the Z/H epilogue for the Z GEMM.
 #define COLA_DEFINE_LAUNCHERS
 #include "gemm_launch.cuh"
 
@@ -170,9 +170,9 @@ template cudaError_t launch_gemm<256, 1, true, true, EPI_TAIL>(const GemmBatch&,
 template cudaError_t launch_gemm<128, 2, true, true, EPI_TAIL>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<256, 1, true, true, EPI_TAIL, true>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<128, 1, true, true, EPI_STORE>(const GemmBatch&, int, bool, cudaStream_t);
-// split-K output GEMMs of small launches (both operands K-major)
+// split-K output GEMMs of small launches (both operands K-major; so few tiles
+// that fill_bn takes 128 columns)
 template cudaError_t launch_gemm<128, 1, false, false, EPI_F32>(const GemmBatch&, int, bool, cudaStream_t);
-template cudaError_t launch_gemm<256, 1, false, false, EPI_F32>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<256, 1, true, true, EPI_STORE>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<128, 2, true, true, EPI_STORE>(const GemmBatch&, int, bool, cudaStream_t);
 template cudaError_t launch_gemm<256, 1, true, true, EPI_STORE, true>(const GemmBatch&, int, bool, cudaStream_t);

@@ -235,13 +235,14 @@ void set_splits(GemmParams& p, int S)
     p.units = p.m_tiles * p.n_tiles * p.splits;
 }
 
-// Split-K for the forward GEMMs of small launches: with fewer output tiles
-// than half the SMs (a few hundred tokens or less) and K >= 1024, the K range
-// of each tile is split (>= 4 k-blocks per split, up to about one unit per
-// SM); the fp32 partials are reduced, and the epilogue applied, by the reduce
-// kernel.  A shorter K streams too little per tile for the extra reduce
-// launch to pay off (measured: the 2048-token 60M layer, K = 512 / 128, got
-// slower).  1 = no split.
+// Split-K through fp32 slabs for the forward GEMMs of small launches: with fewer
+// output tiles than half the SMs (a few hundred tokens or less) and K >= 1024,
+// the K range of each tile is split (>= 4 k-blocks per split, up to about one
+// unit per SM); the fp32 partials are reduced, and the epilogue applied, by the
+// reduce kernel.  The Y GEMMs of r >= 1024 above 64 tokens, and the Z/H GEMMs
+// while the cluster reduction (rank_gemm_splits) is switched off.  A shorter K
+// streams too little per tile for the extra reduce launch to pay off (measured:
+// the 2048-token 60M layer, K = 512 / 128, got slower).  1 = no split.
 int small_launch_splits(int tiles, int k_blocks, int sms)
 {
     if (2 * tiles >= sms || k_blocks < 16) return 1;
@@ -495,8 +496,8 @@ cudaError_t dispatch_sig(int bn, int msub, GemmBatch& b, int sms, cudaStream_t s
     b.units = units;
     const bool pdl = flops < 64e9;
     // the split-K forward GEMMs of small launches (K-major fp32 partials) run
-    // on single-CTA 128-row tiles only; the gated dX GEMM on CTA pairs or on
-    // 128 x 128 tiles (its long-K form on pairs only)
+    // on 128 x 128 tiles only; the gated dX GEMM on CTA pairs or on 128 x 128
+    // tiles (its long-K form on pairs only)
     constexpr bool small_only = EPI == EPI_F32 && !A_MN;
     constexpr bool glu_bwd = epi_glu_bwd(EPI);
     if constexpr (!small_only && EPI != EPI_STORE64) {
@@ -508,7 +509,7 @@ cudaError_t dispatch_sig(int bn, int msub, GemmBatch& b, int sms, cudaStream_t s
     // planned tiles exist as above and below only
     if (msub != 1 && (bn == 256 || small_only || glu_bwd)) return cudaErrorInvalidValue;
     const int grid = units < sms ? units : sms;
-    if constexpr (glu_bwd) {
+    if constexpr (glu_bwd || small_only) {
         if (bn == 256) return cudaErrorInvalidValue;
     } else {
         if (bn == 256) return launch_gemm<256, 1, A_MN, B_MN, EPI, false, SIG>(b, grid, pdl, s);

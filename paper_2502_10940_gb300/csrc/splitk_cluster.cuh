@@ -5,8 +5,8 @@
 //   D[tile] = sum over s = 0..S-1 of  sum over k of split s of  P[m, k] Q[n, k]
 //
 // the weight gradients (dB = dY^T H, dA = dZ^T X, Sec. 3.4: k = tokens, P and Q
-// token-major, read MN-major), Z = X A^T with H = sigma(Z) (both K-major),
-// dZ = (dY B) * sigma'(Z) (B read MN-major) and Y = H B^T (both K-major).
+// token-major, read MN-major), Z = X A^T with H = sigma(Z) (both K-major) and
+// dZ = (dY B) * sigma'(Z) (B read MN-major).
 //
 // Each 128 x 128 output tile runs on one cluster of S CTAs (1 <= S <= 8),
 // CTA s accumulating the k-blocks of split s in its own TMEM.  The partial

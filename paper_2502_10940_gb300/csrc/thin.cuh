@@ -30,8 +30,8 @@
 // the main loop's) this follows.
 //
 // Measured (graph-replayed blocks, against the token-major GEMMs with fp32 slabs
-// and reduce launches): 1B-shaped, 32 tokens 57.4 -> 44 us (12 -> 8 launches);
-// 7B-shaped, 1 token 83 -> 58 us (14 -> 8), 16 tokens 82 -> 62 us.  A launch of
+// and reduce launches): 1B-shaped, 32 tokens 57.4 -> 45.5 us (12 -> 8
+// launches); 7B-shaped, 1 token 83 -> 58 us (14 -> 8), 16 tokens 82 -> 62 us.  A launch of
 // the 1B-shaped o layer takes 4.5 us: 0.5 us from the wait to the first k-block,
 // 0.5 us main loop, 1 us staging and exchange, 0.5 us sums and stores, 1.3 us
 // until the next kernel's wait returns; 7B-shaped ones stream their weights at
