@@ -646,6 +646,21 @@ __device__ __forceinline__ void store_row8(__nv_bfloat16* d, const uint4& w, int
         if (e < valid) d16[e] = static_cast<uint16_t>((e & 1) ? (v[e >> 1] >> 16) : (v[e >> 1] & 0xFFFFu));
 }
 
+// Store the 32 x 64 box staged by stage_row128 at `box` to rows of pitch ld at d
+// (its first entry), clipped to `rows` rows and `valid` columns: 128 contiguous
+// bytes of four rows an instruction.  For the chunk that holds a ragged right edge
+// (N % 8 != 0), where a TMA store would write the row padding.  (Each thread
+// storing its own row: Y of 65536 x 1463, r = 256 64 us, this 61; gated forward of
+// 65536 x 1373, r = 128 124 and 121.)
+__device__ __forceinline__ void store_box_clipped(uint32_t box, int lane, __nv_bfloat16* d, long long ld, int rows,
+                                                  int valid)
+{
+    const int j = lane & 7;
+#pragma unroll 1
+    for (int r = lane >> 3; r < 32 && r < rows; r += 4)
+        store_row8(d + r * ld + 8 * j, ld_shared_v4(box + r * 128 + ((j ^ (r & 7)) << 4)), valid - 8 * j);
+}
+
 // The UMMA descriptor of an operand tile at shared-memory address `saddr`
 // (K-major, or MN-major as 64 x 64 boxes 8 KB apart), as two words: every k-step
 // and stage of the ring changes only the address field in the low one, so the
@@ -1175,6 +1190,25 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const int row0 = m_blk * TILE_M + row_off + sub * BM + q * 32;
             const int row = row0 + lane;
             const int nch = chunk_count(x);
+            if constexpr (EPI == EPI_GLU || STORE64) {
+                // a row that does not begin or end on a 32-byte sector writes part of
+                // one there: fetched into L2 ahead, such a sector is not filled from
+                // HBM when it is evicted (gated forward of 65536 x 1373, r = 128 118 ->
+                // 105 us, 65536 x 5461, r = 512 691 -> 681; Y of 32768 x 2733 58 -> 56)
+                const int c0 = n_blk * BN;
+                if (c_first == 0 && row < p.M && (c0 == 0 || c0 + BN >= p.N)) {
+                    auto hint = [&](const __nv_bfloat16* d) {
+                        const __nv_bfloat16* at = d + row * p.d_ld;
+                        if (c0 == 0 && (reinterpret_cast<uint64_t>(at) & 31)) prefetch_l2(at);
+                        if (c0 + BN >= p.N && (reinterpret_cast<uint64_t>(at + p.N) & 31)) prefetch_l2(at + p.N - 1);
+                    };
+                    hint(p.d_ptr);
+                    if (EPI == EPI_GLU && p.has_d2) {
+                        hint(p.d2_ptr);
+                        hint(p.d3_ptr);
+                    }
+                }
+            }
             if (!wait_bounded(&tfull_bar[buf], bphase, wc, ST_TIMEOUT_EPILOGUE)) break;
             tc_fence_after();
             const uint32_t tbase = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
@@ -1229,35 +1263,23 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         auto m = [&](int j) { return mul_bf16x2(g[i][j], u[j]); };
                         auto yg = [&](int j) { return g[i][j]; };
                         auto yu = [&](int j) { return u[j]; };
-                        if ((p.N & 7) != 0 && valid < GLU_COLS) {
-                            // a TMA store would write the row padding past a ragged right edge
-                            if (row < p.M) {
-                                const long long off = row * p.d_ld + col0;
-#pragma unroll
-                                for (int j = 0; j < GLU_COLS / 8; ++j) {
-                                    auto at = [&](auto&& w) {
-                                        return make_uint4(w(4 * j), w(4 * j + 1), w(4 * j + 2), w(4 * j + 3));
-                                    };
-                                    store_row8(p.d_ptr + off + 8 * j, at(m), valid - 8 * j);
-                                    if (p.has_d2) {
-                                        store_row8(p.d2_ptr + off + 8 * j, at(yg), valid - 8 * j);
-                                        store_row8(p.d3_ptr + off + 8 * j, at(yu), valid - 8 * j);
-                                    }
-                                }
-                            }
-                        } else {
-                            auto emit64 = [&](const CUtensorMap* map, auto&& w) {
-                                if (lane == 0) bulk_wait_group_read<0>();   // the box's previous store has read it
+                        const bool ragged = (p.N & 7) != 0 && valid < GLU_COLS;
+                        auto emit64 = [&](const CUtensorMap* map, __nv_bfloat16* d, auto&& w) {
+                            if (lane == 0) bulk_wait_group_read<0>();   // the box's previous store has read it
+                            __syncwarp();
+                            stage_row128(ep, lane, w);
+                            if (ragged) {
                                 __syncwarp();
-                                stage_row128(ep, lane, w);
+                                store_box_clipped(ep, lane, d + row0 * p.d_ld + col0, p.d_ld, p.M - row0, valid);
+                            } else {
                                 fence_proxy_async_smem();
                                 store_box(map, ep, col0, row0);
-                            };
-                            emit64(map_d, m);
-                            if (p.has_d2) {
-                                emit64(map_d2, yg);
-                                emit64(&batch.prob[x.g].map_d3, yu);
                             }
+                        };
+                        emit64(map_d, p.d_ptr, m);
+                        if (p.has_d2) {
+                            emit64(map_d2, p.d2_ptr, yg);
+                            emit64(&batch.prob[x.g].map_d3, p.d3_ptr, yu);
                         }
                     }
                 }
@@ -1288,18 +1310,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 };
                 auto store = [&](int c, const uint32_t (&w)[32]) {
                     const int col0 = n_blk * BN + c * GLU_COLS, valid = p.N - col0;
+                    if (lane == 0) bulk_wait_group_read<0>();
+                    __syncwarp();
+                    stage_row128(ep, lane, [&](int j) { return w[j]; });
                     if ((p.N & 7) != 0 && valid < GLU_COLS) {
-                        // a TMA store would write the row padding past a ragged right edge
-                        if (row < p.M) {
-#pragma unroll
-                            for (int j = 0; j < GLU_COLS / 8; ++j)
-                                store_row8(p.d_ptr + row * p.d_ld + col0 + 8 * j,
-                                           make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]), valid - 8 * j);
-                        }
-                    } else {
-                        if (lane == 0) bulk_wait_group_read<0>();
                         __syncwarp();
-                        stage_row128(ep, lane, [&](int j) { return w[j]; });
+                        store_box_clipped(ep, lane, p.d_ptr + row0 * p.d_ld + col0, p.d_ld, p.M - row0, valid);
+                    } else {
                         fence_proxy_async_smem();
                         store_box(map_d, ep, col0, row0);
                     }
