@@ -808,7 +808,7 @@ cola_status_t run_f2(const Shape& s, int count, const void* const* H, int64_t ld
                                    [&] { return launch_splitk_reduce(rb, st); }));
         }
     }
-    const bool wide = store_boxes64(ms == TILE_PAIR, s.ld_y, count * s.n * s.d_out * 2);
+    const bool wide = store_boxes64(ms == TILE_PAIR, s.d_out, s.ld_y);
     for (int j = 0; j < count; ++j) {
         pr[j].p = base_params(s.n, s.d_out, s.r, bn, ms);
         COLA_MAP(map_kmajor(&pr[j].map_a, H[j], s.r, s.n, ldh, a_box_rows(ms)));
@@ -1079,7 +1079,7 @@ cola_status_t run_b4(const Shape& s, int64_t K, const void* dZ, int64_t ldz, con
 {
     const int bn = fill_bn(s.n, s.d_in, K, 1, sms);
     const int ms = choose_msub(s.n, s.d_in, K, bn);
-    const bool wide = store_boxes64(ms == TILE_PAIR, s.ld_x, s.n * s.d_in * 2);
+    const bool wide = store_boxes64(ms == TILE_PAIR, s.d_in, s.ld_x);
     GemmProblem pr;
     std::memset(&pr, 0, sizeof pr);
     pr.p = base_params(s.n, s.d_in, K, bn, ms);

@@ -143,17 +143,19 @@ int fill_bn(int64_t M, int64_t N, int64_t K, int count, int sms)
     return count * ((M + BM - 1) / BM) * ((N + 127) / 128) <= sms ? 128 : 256;
 }
 
-// Whether plain outputs of pitch `ld` (`bytes` of them in the launch) are stored
-// through 64-column boxes (EPI_STORE64, and EPI_STORE on CTA pairs) or through
-// rings of 32-column ones.  64 columns where rows are not 128-byte aligned (a
-// 64-byte row piece then touches a sector more, twice as often): Y of 110691 x
-// 1463, two of them, 297 -> 222 us; and for outputs that L2 takes: Y of 65536 x
-// 512 20.8 -> 19 us.  Larger aligned outputs are bound by HBM writes, which the
-// ring keeps more of in flight: three of 131072 x 1024 199 us with 64 columns,
-// 194 with 32.
-bool store_boxes64(bool pair, int64_t ld, int64_t bytes)
+// Whether plain outputs of N columns and pitch `ld` are stored through 64-column
+// boxes (EPI_STORE64, and EPI_STORE on CTA pairs) or through rings of 32-column
+// ones.  64 columns where rows are not 32-byte aligned (a 64-byte row piece then
+// touches a sector more, twice as often), 32 against 64: Y of 110691 x 1463, two of
+// them, 306 -> 213 us; 106705 x 712, r = 64, two 98 -> 82; 4047 x 1611, three 15.5 ->
+// 14.4; and for a ragged right edge (N % 8 != 0), which they store by coalesced rows
+// and the ring one element at a time: 65536 x 1021, r = 256 102 -> 54 us.  Other rows
+// are written faster by the ring, which keeps more stores in flight, 64 against 32:
+// 106705 x 720, r = 64, two 69 -> 65 us; 8143 x 1536, three 23.5 -> 23.0; 2048 x
+// 4096, K = 512 12.0 -> 11.7 (but 106705 x 720, one 32 -> 34.6).
+bool store_boxes64(bool pair, int64_t N, int64_t ld)
 {
-    return pair || ld % 64 != 0 || bytes <= (96ll << 20);
+    return pair || ld % 16 != 0 || N % 8 != 0;
 }
 
 // Tile modes ("msub" below): 1 = one CTA runs a 128-row tile; 2 = one CTA
