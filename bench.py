@@ -312,12 +312,12 @@ def launch_cost(kind, shapes, splits, flags):
             b = e * (m * k + n * k + m * n * (3 if flags & 1 else 1))   # M (+ Y_gate, Y_up)
         elif kind == "reduce":
             b = e * m * n * (2 if flags & 1 else 1)   # flag: the Z/H reduce writes Z and H
-        elif kind == "sigma":
+        elif kind in ("sigma", "repack"):
             b = e * 2 * m * n
         else:
             b = 0
         tb += b
-        tf += 0.0 if kind in ("reduce", "sigma") else 2.0 * m * n * k
+        tf += 0.0 if kind in ("reduce", "sigma", "repack") else 2.0 * m * n * k
     return tb, tf
 
 

@@ -129,7 +129,9 @@ cola_status_t cola_workspace_init(void* ws, void* stream);
  * the H of its 128-row tile in shared memory between the two products (H is an
  * intermediate of Eq. (main-fwd), not an output), storing Z and H only as the
  * mode saves them; the results are the same bit for bit
- * (cola_set_fused_forward). */
+ * (cola_set_fused_forward).  Large GEMMs whose A has rows that do not begin on
+ * 32-byte sectors (ld_a % 16 != 0) first copy it to an aligned pitch in the
+ * workspace, where it has room (the training modes; dX too). */
 cola_status_t cola_fwd(const cola_desc_t* desc, const void* X, const void* A, const void* B, void* Y,
                        void* Z_save, void* H_save, void* ws, size_t ws_bytes, void* stream);
 
@@ -370,8 +372,10 @@ typedef enum {
     COLA_KERNEL_FWD_GLU = 7,     /* M = (H_gate B_gate^T) * (H_up B_up^T) (M=n, N=d_ff, K=2r) */
     COLA_KERNEL_FWD_FUSED = 8,   /* Z, H = sigma(Z), Y = H B^T in one kernel, count 2:
                                     (n, r, d_in) and (n, d_out, r) */
-    COLA_KERNEL_BWD_FUSED = 9    /* dZ = (dY B) * sigma'(Z), dX = dZ A in one kernel, count 2:
+    COLA_KERNEL_BWD_FUSED = 9,   /* dZ = (dY B) * sigma'(Z), dX = dZ A in one kernel, count 2:
                                     (n, r, d_out) and (n, d_in, r) */
+    COLA_KERNEL_REPACK = 10      /* A copied to an aligned pitch in the workspace, ahead of a large
+                                    GEMM that reads it            (M=rows, N=d_in, K=0) */
 } cola_kernel_t;
 
 typedef struct {

@@ -31,7 +31,7 @@ SYMBOLS = ("cola_workspace_size", "cola_workspace_init", "cola_fwd", "cola_bwd",
            "cola_status_string")
 STATIC_SCRATCH_BYTES = 64 * 1024 * 1024
 KERNELS = {0: "fwd_zh", 1: "fwd_y", 2: "bwd_dz", 3: "wgrad", 4: "reduce", 5: "bwd_dx", 6: "sigma", 7: "fwd_glu", 8: "fwd_fused",
-           9: "bwd_fused"}
+           9: "bwd_fused", 10: "repack"}
 
 
 class ColaError(RuntimeError):

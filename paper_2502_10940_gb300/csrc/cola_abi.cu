@@ -453,6 +453,56 @@ cola_status_t run_cluster_rank(int op, int sigma, int count, int64_t n, int64_t 
 bool fused_fwd_form(const Shape& s, int sms);
 bool fused_bwd_form(const Shape& s, int sms);
 
+// The weight A [R x d_in] of a large GEMM on CTA pairs at a 128-byte aligned pitch:
+// where its rows do not begin on 32-byte sectors, it is copied into `room` (a part
+// of the workspace that nothing else uses meanwhile; when it is too small A stays
+// where it is), and *A and s->ld_a become the copy's.  Every CTA walks all of A for
+// each of its tiles, and a 128-byte row of a TMA box that straddles sectors and
+// lines costs L2 a second request each time.  Measured, pitch 5464 against 5504
+// (r = 512): Z of 65536 tokens 295 -> 236 us, dX 283 -> 248; with 32-byte aligned
+// rows 8 us to nothing.  The copy (5.6 MB) costs 4 us, so it is made from
+// `min_flops` of that GEMM on.  Passes with it and without: forward, 131072
+// tokens, pitch 1000, r = 256 (67 GFLOP) 152 -> 144 us, 12000 tokens, 4104, r = 512
+// (50) 70 -> 62.5, 8192 tokens (34) 40 -> 36.4, 10000, 1720, r = 768 (26) 50.9 ->
+// 49.5, 16000, 2008, r = 320 (21) the same; backward, 16384 tokens, 4104 (69) 152 ->
+// 147, 12000 (50) and 8192 (34) the same.
+constexpr double ALIGN_FWD_FLOPS = 24e9;
+constexpr double ALIGN_DX_FLOPS = 60e9;
+
+cola_status_t align_weight(Shape* s, int64_t R, const void** A, int64_t K, int64_t N, double min_flops, void* room,
+                           size_t room_bytes, int sms, cudaStream_t st)
+{
+    const int64_t ld = (s->d_in + 63) / 64 * 64;
+    if (s->ld_a % 16 == 0 || 2.0 * s->n * N * K < min_flops) return COLA_OK;
+    if (choose_msub(s->n, N, K, choose_bn_for(s->n, N, K)) != TILE_PAIR) return COLA_OK;
+    if (static_cast<size_t>(R) * ld * 2 > room_bytes) return COLA_OK;
+    const int64_t mnk[1][3] = {{R, s->d_in, 0}};
+    COLA_TRY(launched(traced(COLA_KERNEL_REPACK, 1, mnk, 1, 0, st, [&] {
+        return launch_repack(*A, s->ld_a, room, ld, R, static_cast<int>(s->d_in), sms, st);
+    })));
+    *A = room;
+    s->ld_a = ld;
+    return COLA_OK;
+}
+
+// Of a training forward, whose workspace holds a dZ that only the backward uses.
+cola_status_t align_fwd_weight(const cola_desc_t& d, Shape* s, int64_t R, const void** A, void* dZ, int sms,
+                               cudaStream_t st)
+{
+    const size_t room = d.mode != COLA_MODE_INFER ? static_cast<size_t>(s->n) * R * 2 : 0;
+    return align_weight(s, R, A, s->d_in, R, ALIGN_FWD_FLOPS, dZ, room, sms, st);
+}
+
+// Of the plain dX GEMM (the gated one is bound by its epilogue: 592 -> 588 us),
+// after the weight gradients: they are done with the partials and, under CoLA-M,
+// with the H before them.
+cola_status_t align_bwd_weight(const cola_desc_t& d, Shape* s, int64_t R, const void** A, void* ws, const WsLayout& L,
+                               int sms, cudaStream_t st)
+{
+    const size_t off = d.mode == COLA_MODE_COLA_M ? L.h_off : L.part_off;
+    return align_weight(s, R, A, R, s->d_in, ALIGN_DX_FLOPS, wsb(ws) + off, L.total - off, sms, st);
+}
+
 // F1: Z = X A^T, H = sigma(Z)  (N = r, or 3r for the fused q/k/v factors;
 // Z / H pitch ldz)
 cola_status_t run_f1(const Shape& s, int sigma, int64_t N, const void* X, const void* A, void* Z, void* H,
@@ -1146,6 +1196,7 @@ cola_status_t cola_fwd(const cola_desc_t* desc, const void* X, const void* A, co
         COLA_TRY(run_thin_f1(s, desc->sigma, s.r, X, A, Z_save, H, status, sms, st));
         return run_thin_f2(s, 1, H, s.r, Bs, Ys, status, sms, st);
     }
+    COLA_TRY(align_fwd_weight(*desc, &s, s.r, &A, wsb(ws) + L.dz_off, sms, st));
     COLA_TRY(run_f1(s, desc->sigma, s.r, X, A, Z_save, H, s.r, part, part_bytes, status, sms, st));
     return run_f2(s, 1, Hs, s.r, Bs, Ys, part, part_bytes, status, sms, st);
 }
@@ -1205,6 +1256,7 @@ cola_status_t bwd_single(const cola_desc_t* desc, const void* X, const void* A, 
     COLA_TRY(run_b1(s, desc->sigma, 1, dYs, Bs, Zs, s.r, dZs, cola_m ? Hs : nullptr, status, sms, st));
     COLA_TRY(run_wgrad(w, s.n, jobs, desc->wgrad_fp32, part, part_bytes, status, sms, st));
     if (glu) return run_b4_glu(s, s.r, dZ, s.r, A, glu->Yg, glu->Yu, glu->dYg, glu->dYu, status, sms, st);
+    COLA_TRY(align_bwd_weight(*desc, &s, s.r, &A, ws, L, sms, st));
     return run_b4(s, s.r, dZ, s.r, A, dX, status, sms, st);
 }
 
@@ -1254,6 +1306,7 @@ cola_status_t cola_fwd_gate_up(const cola_desc_t* desc, const void* X, const voi
         COLA_TRY(run_thin_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, status, sms, st));
         return run_thin_glu(s, H, B_gate, B_up, M, Y_gate, Y_up, status, sms, st);
     }
+    COLA_TRY(align_fwd_weight(*desc, &s, R, &A_cat, wsb(ws) + L.dz_off, sms, st));
     COLA_TRY(run_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, R, part, part_bytes, status, sms, st));
     return run_glu(s, H, R, B_gate, B_up, M, Y_gate, Y_up, status, sms, st);
 }
@@ -1283,6 +1336,7 @@ cola_status_t cola_fwd_shared_x(const cola_desc_t* desc, int32_t count, const vo
         COLA_TRY(run_thin_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, status, sms, st));
         return run_thin_f2(s, count, H, R, B, Y, status, sms, st);
     }
+    COLA_TRY(align_fwd_weight(*desc, &s, R, &A_cat, wsb(ws) + L.dz_off, sms, st));
     COLA_TRY(run_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, R, part, part_bytes, status, sms, st));
     const void* Hs[3] = {H, H + slice, H + 2 * slice};
     return run_f2(s, count, Hs, R, B, Y, part, part_bytes, status, sms, st);
@@ -1329,6 +1383,7 @@ cola_status_t cola_bwd_shared_x(const cola_desc_t* desc, int32_t count, const vo
     COLA_TRY(run_b1(s, desc->sigma, count, dY, B, Zs, R, dZs, cola_m ? Hr : nullptr, status, sms, st));
     const WgradPlan w = wgrad_plan(*desc, count, sms);
     COLA_TRY(run_wgrad(w, s.n, jobs, desc->wgrad_fp32, part, part_bytes, status, sms, st));
+    COLA_TRY(align_bwd_weight(*desc, &s, R, &A_cat, ws, L, sms, st));
     return run_b4(s, R, dZ, R, A_cat, dX, status, sms, st);
 }
 

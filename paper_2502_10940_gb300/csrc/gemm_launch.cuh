@@ -72,6 +72,9 @@ cudaError_t launch_tail_reduce(const TailReduce& r, int sms, cudaStream_t stream
 // H = bf16(sigma(Z)) elementwise over `elems` bf16 values (a multiple of 8;
 // both pointers 16-byte aligned).
 cudaError_t launch_sigma(const void* Z, void* H, long long elems, int sigma, int sms, cudaStream_t stream);
+// `rows` rows of `cols` bf16 from pitch ld_s to pitch ld_d
+cudaError_t launch_repack(const void* src, long long ld_s, void* dst, long long ld_d, long long rows, int cols, int sms,
+                          cudaStream_t stream);
 
 #ifdef COLA_DEFINE_LAUNCHERS
 template <int BN, int MSUB, bool A_MN, bool B_MN, int EPI, bool PAIR, int SIG>
