@@ -453,28 +453,36 @@ cola_status_t run_cluster_rank(int op, int sigma, int count, int64_t n, int64_t 
 bool fused_fwd_form(const Shape& s, int sms);
 bool fused_bwd_form(const Shape& s, int sms);
 
-// The weight A [R x d_in] of a large GEMM on CTA pairs at a 128-byte aligned pitch:
-// where its rows do not begin on 32-byte sectors, it is copied into `room` (a part
-// of the workspace that nothing else uses meanwhile; when it is too small A stays
-// where it is), and *A and s->ld_a become the copy's.  Every CTA walks all of A for
-// each of its tiles, and a 128-byte row of a TMA box that straddles sectors and
-// lines costs L2 a second request each time.  Measured, pitch 5464 against 5504
-// (r = 512): Z of 65536 tokens 295 -> 236 us, dX 283 -> 248; with 32-byte aligned
-// rows 8 us to nothing.  The copy (5.6 MB) costs 4 us, so it is made from
-// `min_flops` of that GEMM on.  Passes with it and without: forward, 131072
-// tokens, pitch 1000, r = 256 (67 GFLOP) 152 -> 144 us, 12000 tokens, 4104, r = 512
-// (50) 70 -> 62.5, 8192 tokens (34) 40 -> 36.4, 10000, 1720, r = 768 (26) 50.9 ->
-// 49.5, 16000, 2008, r = 320 (21) the same; backward, 16384 tokens, 4104 (69) 152 ->
-// 147, 12000 (50) and 8192 (34) the same.
-constexpr double ALIGN_FWD_FLOPS = 24e9;
-constexpr double ALIGN_DX_FLOPS = 60e9;
+// The weight A [R x d_in] of a large GEMM at a 128-byte aligned pitch: where its
+// rows do not begin on 32-byte sectors, it is copied into `room` (a part of the
+// workspace that nothing else uses meanwhile; when it is too small A stays where it
+// is), and *A and s->ld_a become the copy's.  Every CTA walks A for each of its
+// tiles, and a 128-byte row of a TMA box that straddles sectors and lines costs L2
+// a second request each time.  Measured, pitch 5464 against 5504 (r = 512): Z of
+// 65536 tokens 295 -> 236 us, dX 283 -> 248; with 32-byte aligned rows 8 us to
+// nothing.  The copy takes 2 (256 KB) to 4 us (5.6 MB), so it is made from so many
+// FLOP of the GEMM on.  Passes with it and without, CTA pairs: forward, 12000 tokens,
+// pitch 4104, r = 512 (50 GFLOP) 70 -> 62.5 us, 8192 tokens (34) 40 -> 36.4, 10000,
+// 1720, r = 768 (26) 50.9 -> 49.5, 16000, 2008, r = 320 (21) the same; backward, 16384
+// tokens, 4104 (69) 152 -> 147, 12000 (50) and 8192 (34) the same.  Single CTAs (of
+// launches with many row tiles): forward, 131072 tokens, 1000, r = 128 (34) 101.5 ->
+// 87.3, 20000, 2008, r = 192 (15) 58.5 -> 52.2, 65536, 520, r = 128 (9) 68.8 -> 64.4,
+// 30000 (4) the same; backward 202 -> 196, 92.2 -> 89.9, 120.1 -> 120.5, the same.
+struct AlignRule {
+    double pair_flops, single_flops;
+};
+constexpr AlignRule ALIGN_FWD{24e9, 8e9};
+constexpr AlignRule ALIGN_DX{60e9, 12e9};
+constexpr int64_t ALIGN_SINGLE_TOKENS = 8192;
 
-cola_status_t align_weight(Shape* s, int64_t R, const void** A, int64_t K, int64_t N, double min_flops, void* room,
-                           size_t room_bytes, int sms, cudaStream_t st)
+cola_status_t align_weight(Shape* s, int64_t R, const void** A, int64_t K, int64_t N, const AlignRule& rule,
+                           void* room, size_t room_bytes, int sms, cudaStream_t st)
 {
     const int64_t ld = (s->d_in + 63) / 64 * 64;
-    if (s->ld_a % 16 == 0 || 2.0 * s->n * N * K < min_flops) return COLA_OK;
-    if (choose_msub(s->n, N, K, choose_bn_for(s->n, N, K)) != TILE_PAIR) return COLA_OK;
+    if (s->ld_a % 16 == 0) return COLA_OK;
+    const bool pair = choose_msub(s->n, N, K, choose_bn_for(s->n, N, K)) == TILE_PAIR;
+    if (2.0 * s->n * N * K < (pair ? rule.pair_flops : rule.single_flops)) return COLA_OK;
+    if (!pair && s->n < ALIGN_SINGLE_TOKENS) return COLA_OK;
     if (static_cast<size_t>(R) * ld * 2 > room_bytes) return COLA_OK;
     const int64_t mnk[1][3] = {{R, s->d_in, 0}};
     COLA_TRY(launched(traced(COLA_KERNEL_REPACK, 1, mnk, 1, 0, st, [&] {
@@ -490,7 +498,7 @@ cola_status_t align_fwd_weight(const cola_desc_t& d, Shape* s, int64_t R, const 
                                cudaStream_t st)
 {
     const size_t room = d.mode != COLA_MODE_INFER ? static_cast<size_t>(s->n) * R * 2 : 0;
-    return align_weight(s, R, A, s->d_in, R, ALIGN_FWD_FLOPS, dZ, room, sms, st);
+    return align_weight(s, R, A, s->d_in, R, ALIGN_FWD, dZ, room, sms, st);
 }
 
 // Of the plain dX GEMM (the gated one is bound by its epilogue: 592 -> 588 us),
@@ -500,7 +508,7 @@ cola_status_t align_bwd_weight(const cola_desc_t& d, Shape* s, int64_t R, const 
                                int sms, cudaStream_t st)
 {
     const size_t off = d.mode == COLA_MODE_COLA_M ? L.h_off : L.part_off;
-    return align_weight(s, R, A, R, s->d_in, ALIGN_DX_FLOPS, wsb(ws) + off, L.total - off, sms, st);
+    return align_weight(s, R, A, R, s->d_in, ALIGN_DX, wsb(ws) + off, L.total - off, sms, st);
 }
 
 // F1: Z = X A^T, H = sigma(Z)  (N = r, or 3r for the fused q/k/v factors;

@@ -21,9 +21,10 @@ def _cuda():
 
 # n, d_in, r, projections (0: the down layer of a gated MLP, forward only): d_in inside and at the
 # end of a 16-byte group; token splits of the weight gradients that leave room for
-# the copy; a token count whose dZ has none
+# the copy; a token count whose dZ has none; single CTAs
 @pytest.mark.parametrize("n,d_in,r,c", [(16385, 4101, 512, 1), (9000, 4104, 512, 2), (16400, 4099, 512, 0),
-                                        (65536, 1000, 512, 1), (2048, 33000, 512, 1)])
+                                        (65536, 1000, 512, 1), (2048, 33000, 512, 1), (30001, 1000, 256, 1),
+                                        (24000, 997, 128, 3)])
 @pytest.mark.parametrize("mode", ["cola", "cola_m"])
 def test_misaligned_weight(n, d_in, r, c, mode):
     from paper_2502_10940_gb300 import cola
