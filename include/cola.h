@@ -107,7 +107,9 @@ typedef struct {
  * cola_bwd, 2 or 3 for cola_fwd_shared_x / cola_bwd_shared_x with that count
  * (3 for the q/k/v entry points).  The value depends on n, r, d_in, d_out,
  * the mode, wgrad_fp32 and the device's SM count (it sizes the
- * weight-gradient split over tokens). */
+ * weight-gradient split over tokens), and under COLA_MODE_INFER on ld_a (room
+ * for an aligned copy of A; a workspace of the size for an aligned ld_a is
+ * accepted too, and A then read in place). */
 cola_status_t cola_workspace_size(const cola_desc_t* desc, int32_t nproj, size_t* bytes);
 
 /* Zero the workspace status word (first 256 bytes of ws), asynchronously. */
@@ -131,7 +133,7 @@ cola_status_t cola_workspace_init(void* ws, void* stream);
  * mode saves them; the results are the same bit for bit
  * (cola_set_fused_forward).  Large GEMMs whose A has rows that do not begin on
  * 32-byte sectors (ld_a % 16 != 0) first copy it to an aligned pitch in the
- * workspace, where it has room (the training modes; dX too). */
+ * workspace, where it has room (dX too). */
 cola_status_t cola_fwd(const cola_desc_t* desc, const void* X, const void* A, const void* B, void* Y,
                        void* Z_save, void* H_save, void* ws, size_t ws_bytes, void* stream);
 

@@ -71,3 +71,33 @@ def test_misaligned_weight(n, d_in, r, c, mode):
     assert torch.equal(torch.as_strided(A0, (c * r, lx), (lx, 1)), A0_bits)
     dA = got[c + 3]
     assert (torch.as_strided(dA, (c * r, lx), (lx, 1))[:, d_in:] == 0).all()
+
+
+# single CTAs and CTA pairs; a workspace with and without the room for the copy
+@pytest.mark.parametrize("n,d_in,r,c", [(30001, 1000, 256, 1), (9000, 4101, 512, 2)])
+def test_misaligned_weight_inference(n, d_in, r, c):
+    from paper_2502_10940_gb300 import cola
+    lx, la, d_out = I.padded_ld(d_in), (d_in + 63) // 64 * 64, 256
+    X = I.normal_bf16(n, d_in, 1.0, 1, "cuda", ld=lx)
+    A0 = I.normal_bf16(c * r, d_in, d_in ** -0.5, 2, "cuda", ld=lx)
+    A1 = torch.empty((c * r, la), dtype=torch.bfloat16, device="cuda")[:, :d_in].copy_(A0)
+    B = [I.normal_bf16(d_out, r, r ** -0.5, 3 + j, "cuda") for j in range(c)]
+
+    def run(A, less=0):
+        Y = [torch.zeros((n, d_out), dtype=torch.bfloat16, device="cuda") for _ in range(c)]
+        d = cola.desc(n, d_in, d_out, r, ld_x=lx, ld_a=A.stride(0), mode="infer")
+        ws = cola.workspace(d, c)
+        with cola.Trace(8) as tr:
+            if c > 1:
+                cola.cola_fwd_shared_x(d, X, A, B, Y, None, None, ws[:ws.numel() - less])
+            else:
+                cola.cola_fwd(d, X, A, B[0], Y[0], None, None, ws[:ws.numel() - less])
+        assert cola.cola_check_status(ws) == (0, 0)
+        return [t[0] for t in tr.records()].count("repack"), Y, ws.numel()
+
+    k1, want, b1 = run(A1)
+    k0, got, b0 = run(A0)
+    k2, low, _ = run(A0, less=b0 - b1)
+    assert (k0, k1, k2) == (1, 0, 0) and b0 - b1 == (c * r * la * 2 + 255) // 256 * 256
+    assert all(torch.equal(g, w) and torch.equal(x, w) for g, x, w in zip(got, low, want))
+    assert float(want[0].float().norm()) > 0
