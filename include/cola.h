@@ -235,6 +235,8 @@ cola_status_t cola_fwd_gate_up(const cola_desc_t* desc, const void* X, const voi
  * and stores the gradients at the product's factors,
  *     dY_gate = bf16(bf16(dM) * Y_up),   dY_up = bf16(bf16(dM) * Y_gate),
  * which the gate/up backward (cola_bwd_shared_x, count 2) takes as its dY.
+ * dY_gate and dY_up may be written in place, over Y_gate and Y_up (same pointer,
+ * either way round): every element of both is read before a gradient lies over it.
  * dA, dB as in cola_bwd; H_save NULL under COLA_M; ws: cola_workspace_size(desc, 1). */
 cola_status_t cola_bwd_down_gated(const cola_desc_t* desc, const void* M, const void* A, const void* B,
                                   const void* dY, const void* Z_save, const void* H_save, const void* Y_gate,

@@ -1407,13 +1407,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         if (ZSLOTS != 2 && ++zslot_u == ZSLOTS) zslot_u = 0;
                         if (!ok) break;
                         const uint32_t box = ep + b * epi_slot_bytes(EPI);
+                        // the caller may hand Y_gate's storage to dY_gate: its box, in
+                        // flight since a box ago, has landed before dY_gate is stored (in
+                        // a ragged chunk times_dm stores; else the box is, further down)
+                        auto gate_landed = [&]() {
+                            return wait_bounded(&zbar[zslot_u], (zphase >> zslot_u) & 1u, wc, ST_TIMEOUT_EPILOGUE);
+                        };
+                        if (GLU_ONE && f == 0 && ragged) ok = gate_landed();
+                        if (!ok) break;
                         times_dm(box, f == 0 ? p.d_ptr : p.d2_ptr);
                         if (!GLU_ONE) times_dm(box + GLU_BOX_BYTES, p.d2_ptr);
                         if (GLU_ONE) {
                             z_issue();   // two boxes ahead, into the slot stored from a box ago
-                            // the caller may hand Y_gate's storage to dY_gate: its box
-                            // has landed before dY_gate is stored
-                            if (f == 0) ok = wait_bounded(&zbar[zslot_u], (zphase >> zslot_u) & 1u, wc, ST_TIMEOUT_EPILOGUE);
+                            if (f == 0 && !ragged) ok = gate_landed();
                             if (!ok) break;
                         }
                         fence_proxy_async_smem();   // the slot's writes (ragged: reads) before its stores (next load)

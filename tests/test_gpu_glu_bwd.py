@@ -58,3 +58,34 @@ def test_gated_dx_chunk_edges(n, d_ff, r, pair):
     check(wide(None), wide(None))
     check(Yg, Yu)       # in place: dY_gate over Y_gate, dY_up over Y_up
     assert cola.cola_check_status(ws)[0] == 0
+
+
+# d_ff mod 64 = 1, 33, 63: the last chunk of a row is stored directly, not from its box
+@pytest.mark.parametrize("swap", [False, True], ids=["over", "crossed"])
+@pytest.mark.parametrize("n,d_ff,r", [(4360, 4033, 1024), (4330, 4065, 768), (2177, 4095, 1024), (4360, 4095, 512)])
+def test_gated_dx_in_place_at_a_ragged_edge(n, d_ff, r, swap):
+    """Gradients over the saved outputs equal those written apart, bit for bit, run after run."""
+    from paper_2502_10940_gb300 import cola
+    d, ld = 128, I.padded_ld(d_ff)
+    M, Yg, Yu = (I.normal_bf16(n, d_ff, 1.0, s, "cuda", ld=ld) for s in (1, 2, 3))
+    A, B = I.normal_bf16(r, d_ff, d_ff ** -0.5, 4, "cuda", ld=ld), I.normal_bf16(d, r, r ** -0.5, 5, "cuda")
+    dY, Z = I.normal_bf16(n, d, 1.0, 6, "cuda"), I.normal_bf16(n, r, 1.0, 7, "cuda")
+    dd = cola.desc(n, d_ff, d, r, ld_x=ld, ld_a=ld, mode="cola_m")
+    ws = cola.workspace(dd)
+    dA, dB = torch.empty((r, ld), dtype=torch.bfloat16, device="cuda")[:, :d_ff], torch.empty_like(B)
+
+    def run(yg, yu, dyg, dyu):
+        with cola.Trace(8) as tr:
+            cola.cola_bwd_down_gated(dd, M, A, B, dY, Z, None, yg, yu, dyg, dyu, dA, dB, ws)
+        assert [x[3] & 4 for x in tr.records() if x[0] == "bwd_dx"] == [4], tr.records()   # CTA pairs
+        return dyg, dyu
+
+    def fresh(t):
+        return torch.empty((n, ld), dtype=torch.bfloat16, device="cuda")[:, :d_ff].copy_(t)
+
+    want = run(Yg, Yu, fresh(Yg), fresh(Yu))
+    for _ in range(8):
+        yg, yu = fresh(Yg), fresh(Yu)
+        got = run(yg, yu, *((yu, yg) if swap else (yg, yu)))
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    assert cola.cola_check_status(ws)[0] == 0
