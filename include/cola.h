@@ -335,7 +335,7 @@ cola_status_t cola_selftest_wait_timeout_cluster(void* ws, size_t ws_bytes, void
  * COLA_STATIC_SCRATCH_BYTES inside libcola.so, which every GPU that loads
  * the array holds until the process exits.  The entry point calls no
  * cudaMalloc, cudaFree or other allocating routine.  A problem whose fp32
- * partial tile grid (M and N rounded up to the tile size) does not fit the
+ * partial tile grid (M and N rounded up to multiples of 128) does not fit the
  * array even without a token split returns COLA_ERR_WORKSPACE before any
  * launch.  A problem the planner runs without a token split, with a bf16
  * D, stores D straight from the GEMM epilogue and does not touch the array.

@@ -86,13 +86,9 @@ extern "C" cola_status_t cola_wgrad_static_scratch(int64_t n_tokens, int64_t M, 
         return COLA_ERR_LAUNCH;
     if (major != 10 || minor != 3) return COLA_ERR_UNSUPPORTED;
 
-    // ---- plan; shrink the token split until its partials fit the static scratch
-    const int64_t Ms[1] = {M}, Ns[1] = {N};
-    WgradPlan w = plan_wgrad(Ms, Ns, 1, n_tokens, sms);
-    const size_t slab_bytes = static_cast<size_t>(w.slab[0]) * 4;
-    if (slab_bytes > kStaticScratchBytes) return COLA_ERR_WORKSPACE;   // too large even unsplit
-    const int max_splits = static_cast<int>(kStaticScratchBytes / slab_bytes);
-    if (w.p[0].splits > max_splits) set_splits(w.p[0], max_splits);
+    // ---- plan tiles and token split so that the partials fit the static scratch
+    WgradPlan w;
+    if (!plan_wgrad_within(M, N, n_tokens, kStaticScratchBytes, sms, &w)) return COLA_ERR_WORKSPACE;
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     GemmBatch b;

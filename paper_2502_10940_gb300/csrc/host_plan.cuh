@@ -335,26 +335,14 @@ struct WgradPlan {
     double cost;                   // choose_splits' cost of the chosen split
 };
 
-WgradPlan plan_wgrad(const int64_t* M, const int64_t* N, int count, int64_t ntok, int sms)
+// The plan with tiles of bn columns in mode msub.
+WgradPlan plan_wgrad_tiles(const int64_t* M, const int64_t* N, int count, int64_t ntok, int bn, int msub, int sms)
 {
     WgradPlan w;
     std::memset(&w, 0, sizeof w);
     w.count = count;
-    w.bn = 256;
-    for (int i = 0; i < count; ++i) {
-        const int b = choose_bn_for(M[i], N[i], ntok);
-        w.bn = b < w.bn ? b : w.bn;
-    }
-    w.msub = TILE_PAIR;   // the smallest tile any GEMM of the group would take
-    for (int i = 0; i < count; ++i) {
-        const int ms = choose_msub(M[i], N[i], ntok, w.bn);
-        if (ms == 1 || (ms == 2 && w.msub == TILE_PAIR)) w.msub = ms;
-    }
-    if (w.bn == 256 && w.msub == 1) {   // 128 columns where those tiles still run in one wave
-        int64_t t = 0;
-        for (int i = 0; i < count; ++i) t += ((M[i] + BM - 1) / BM) * ((N[i] + 127) / 128);
-        if (t <= sms) w.bn = 128;
-    }
+    w.bn = bn;
+    w.msub = msub;
     int tiles = 0;
     for (int i = 0; i < count; ++i) {
         w.p[i] = base_params(M[i], N[i], ntok, w.bn, w.msub);
@@ -380,6 +368,42 @@ WgradPlan plan_wgrad(const int64_t* M, const int64_t* N, int count, int64_t ntok
         w.cost = static_cast<double>(waves) * (w.p[0].kb_per_split + (w.splits > 1 ? c_part : 0.0)) + REDUCE_LAUNCH_KB;
     }
     return w;
+}
+
+WgradPlan plan_wgrad(const int64_t* M, const int64_t* N, int count, int64_t ntok, int sms)
+{
+    int bn = 256;
+    for (int i = 0; i < count; ++i) {
+        const int b = choose_bn_for(M[i], N[i], ntok);
+        bn = b < bn ? b : bn;
+    }
+    int msub = TILE_PAIR;   // the smallest tile any GEMM of the group would take
+    for (int i = 0; i < count; ++i) {
+        const int ms = choose_msub(M[i], N[i], ntok, bn);
+        if (ms == 1 || (ms == 2 && msub == TILE_PAIR)) msub = ms;
+    }
+    if (bn == 256 && msub == 1) {   // 128 columns where those tiles still run in one wave
+        int64_t t = 0;
+        for (int i = 0; i < count; ++i) t += ((M[i] + BM - 1) / BM) * ((N[i] + 127) / 128);
+        if (t <= sms) bn = 128;
+    }
+    return plan_wgrad_tiles(M, N, count, ntok, bn, msub, sms);
+}
+
+// The plan of one gradient whose partial tile grid has to fit `limit` bytes even
+// unsplit, with the token split reduced until its slabs do.  Wide tiles round M and
+// N up further: when their grid is too large, 128-column tiles, and then 128 x 128
+// ones, whose grid is the smallest.  false: not even that fits.
+bool plan_wgrad_within(int64_t M, int64_t N, int64_t ntok, size_t limit, int sms, WgradPlan* w)
+{
+    const auto slab = [&] { return static_cast<size_t>(w->slab[0]) * 4; };
+    *w = plan_wgrad(&M, &N, 1, ntok, sms);
+    if (slab() > limit) *w = plan_wgrad_tiles(&M, &N, 1, ntok, 128, choose_msub(M, N, ntok, 128), sms);
+    if (slab() > limit) *w = plan_wgrad_tiles(&M, &N, 1, ntok, 128, 1, sms);
+    if (slab() > limit) return false;
+    const int max_splits = static_cast<int>(limit / slab());
+    if (w->p[0].splits > max_splits) set_splits(w->p[0], max_splits);
+    return true;
 }
 
 // Split-tail schedule of a weight-gradient launch with bf16 outputs

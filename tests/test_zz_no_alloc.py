@@ -85,3 +85,25 @@ def test_rejects_problem_beyond_static_scratch(cola):
     with pytest.raises(cola.ColaError) as e:
         cola.cola_wgrad_static_scratch(4096, M, N, t, M, t, N, t, N)
     assert e.value.status == 4                    # COLA_ERR_WORKSPACE, before any launch
+
+
+# Grids of 256-column (256-row) tiles that do not fit the array, of narrower tiles that do:
+# by columns (67.9, 77.9 MB against 63.0, 64.9) and by rows (70.6 MB; 65.6 of 128 x 128 tiles)
+@pytest.mark.parametrize("n,M,N", [(1836, 9443, 1600), (24994, 25146, 515), (498, 1646, 9776)])
+@pytest.mark.parametrize("fp32", [False, True], ids=["bf16", "fp32"])
+def test_runs_what_fits_in_narrower_tiles(cola, n, M, N, fp32):
+    from paper_2502_10940_gb300 import inputs as I
+    P = I.normal_bf16(n, M, 1.0, 1, "cuda", ld=I.padded_ld(M))
+    Q = I.normal_bf16(n, N, n ** -0.5, 2, "cuda", ld=I.padded_ld(N))
+    ld = I.padded_ld(N)
+    buf = torch.full((M, ld), float("nan"), dtype=torch.float32 if fp32 else torch.bfloat16, device="cuda")
+    D = buf[:, :N]
+    if fp32:
+        D.fill_(1.0)
+    cola.cola_wgrad_static_scratch(n, M, N, P, cola.ld_of(P), Q, cola.ld_of(Q), D, ld, accumulate_f32=fp32)
+    ref = P.float().T @ Q.float() + (1.0 if fp32 else 0.0)
+    err = (D.float() - ref).norm() / ref.norm()
+    # fp32: each of the n / 16 accumulation steps is off by at most one ulp, 2^-23 of the sum,
+    # and the reference by a few; bf16: one rounding, 2^-9 / sqrt(3) = 1.1e-3
+    assert err < (n / 16 * 2.0 ** -23 + 2e-6 if fp32 else 3e-3), float(err)
+    assert buf[:, N:].isnan().all()
