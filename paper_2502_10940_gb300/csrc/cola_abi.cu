@@ -526,7 +526,7 @@ cola_status_t align_bwd_weight(const cola_desc_t& d, Shape* s, int64_t R, const 
 cola_status_t run_f1(const Shape& s, int sigma, int64_t N, const void* X, const void* A, void* Z, void* H,
                      int64_t ldz, float* part, size_t part_bytes, unsigned int* status, int sms, cudaStream_t st)
 {
-    const int Sc = rank_gemm_splits(s.n, N, s.d_in, 1, sms);
+    const int Sc = rank_gemm_splits(s.n, N, s.d_in, 1, sigma, sms, false);
     // (a lone layer with the single-kernel form has to match it bit for bit)
     if (Sc > 1 && g_cluster_splitk.load(std::memory_order_relaxed) && !(N == s.r && fused_fwd_form(s, sms))) {
         RankGemm g = {};
@@ -548,9 +548,9 @@ cola_status_t run_f1(const Shape& s, int sigma, int64_t N, const void* X, const 
     COLA_MAP(map_kmajor(&pr.map_b, A, s.d_in, N, s.ld_a, b_box_rows(bn, ms)));
     const int S = ms == 1 ? small_launch_splits(pr.p.m_tiles * pr.p.n_tiles, pr.p.k_blocks, sms) : 1;
     if (S > 1) {
-        // a small launch with the cluster reduction switched off: K split across
-        // CTAs into fp32 partials, then the reduce applies the Z/H epilogue
-        // (Z = bf16(sum), H = bf16(sigma(Z)))
+        // a small launch that no cluster reduces: K split across CTAs into fp32
+        // partials, then the reduce applies the Z/H epilogue (Z = bf16(sum), H =
+        // bf16(sigma(Z)))
         set_splits(pr.p, S);
         const int64_t slab = partial_elems(pr.p, bn, 1);
         if (static_cast<size_t>(pr.p.splits * slab) * 4 > part_bytes) return COLA_ERR_WORKSPACE;
@@ -901,7 +901,7 @@ cola_status_t run_b1(const Shape& s, int sigma, int count, const void* const* dY
                      const void* const* Z, int64_t ldz, void* const* dZ, void* const* Hout, unsigned int* status,
                      int sms, cudaStream_t st)
 {
-    const int Sc = rank_gemm_splits(s.n, s.r, s.d_out, count, sms);
+    const int Sc = rank_gemm_splits(s.n, s.r, s.d_out, count, sigma, sms, true);
     if (Sc > 1 && g_cluster_splitk.load(std::memory_order_relaxed) && !(count == 1 && fused_bwd_form(s, sms))) {
         RankGemm g = {};
         g.ldt = s.ld_y;

@@ -241,8 +241,9 @@ void set_splits(GemmParams& p, int S)
 // output tiles than half the SMs (a few hundred tokens or less) and K >= 1024,
 // the K range of each tile is split (>= 4 k-blocks per split, up to about one
 // unit per SM); the fp32 partials are reduced, and the epilogue applied, by the
-// reduce kernel.  The Y GEMMs of r >= 1024 above 64 tokens, and the Z/H GEMMs
-// while the cluster reduction (rank_gemm_splits) is switched off.  A shorter K
+// reduce kernel.  The Y GEMMs of r >= 1024 above 64 tokens, and the Z/H GEMMs of 33
+// to 64 tokens at r < 256 (but for GELU), or of any number while the cluster
+// reduction (rank_gemm_splits) is switched off.  A shorter K
 // streams too little per tile for the extra reduce launch to pay off (measured:
 // the 2048-token 60M layer, K = 512 / 128, got slower).  1 = no split.
 int small_launch_splits(int tiles, int k_blocks, int sms)
@@ -282,18 +283,38 @@ int cluster_splits(int tiles, int k_blocks, int sms, int* cost = nullptr)
 }
 
 // K splits, inside clusters, of the `count` rank-r GEMMs of one launch (Z of the
-// forward, dZ of the backward): 128 x 128 tiles, fewer than half the SMs, not
+// forward, dZ of the backward): 128 x 128 tiles, at most half as many as SMs, not
 // compute-heavy.  1 = no split.  Measured against fp32 slabs with a reduce launch
 // (Z) and an unsplit dZ, whole graph-replayed passes with the schedules below:
 // q/k/v of 509 tokens, d = 1024, r = 256 23.9 -> 16.4 us forward, 58.8 -> 37.4 us
 // with its backward; a 150-token layer 3000 -> 3000, r = 768 66.1 -> 41.1 us; a
 // 2048-token 350M-shaped block 268 -> 192 us.
-int rank_gemm_splits(int64_t n, int64_t N, int64_t K, int count, int sms)
+//   Z   from K = 1024 on (13 k-blocks with few tiles): shorter ones are no slower
+//       unsplit (forward of 2 to 74 tiles, split against unsplit: 8 k-blocks 1.12 to
+//       1.27, 12 1.04 to 1.21, 13 and 14 0.97 to 1.02 up to 24 tiles and 1.05 to 1.17
+//       above; from 16 on the other way is the slabs', 0.65 to 0.97), and above 64
+//       tokens: with fewer rows the slabs' reduce is the shorter way (one tile of 40
+//       tokens, K = 1024 to 11008 1.05 to 1.11, of 128 tokens 0.88 to 0.95).
+//   dZ  where the split takes enough k-blocks off the longest CTA to pay for the
+//       exchange (whole backward, split against unsplit: 5 fewer 1.00 to 1.04, 8
+//       0.93 to 1.03; in two splits, whose SMs the unsplit tiles half fill, 8 fewer
+//       1.01 to 1.03, 10 1.00), and always up to 64 tokens, of whose rows the exchange
+//       moves few (three of 1 to 9 tokens, K = 576 to 689 0.93 to 0.95).
+// Both hold for SiLU and the identity.  GELU's elementwise work outweighs the
+// exchange, and the splits share it out: split for every K that can be (gated MLP
+// of 783 tokens, 960 -> 2176, r = 192 15.9 -> 14.0 us, 585 tokens, 696 -> 1536, r =
+// 128, two projections 14.9 -> 12.7; 52 tokens, 862 -> 2304 14.0 -> 9.8).
+int rank_gemm_splits(int64_t n, int64_t N, int64_t K, int count, int sigma, int sms, bool dz)
 {
     if (heavy_gemm(n, N, K)) return 1;
     const int64_t tiles = count * ((n + BM - 1) / BM) * ((N + CBN - 1) / CBN);
     if (2 * tiles > sms) return 1;
-    return cluster_splits(static_cast<int>(tiles), static_cast<int>((K + BK - 1) / BK), sms);
+    const int kb = static_cast<int>((K + BK - 1) / BK);
+    const bool cheap = sigma != SIG_GELU;
+    if (cheap && !dz && (n <= THIN_MAX_TOKENS || kb < 13 || (kb < 16 && tiles > 24))) return 1;
+    const int S = cluster_splits(static_cast<int>(tiles), kb, sms);
+    if (cheap && dz && n > THIN_MAX_TOKENS && kb - (kb + S - 1) / S < (S == 2 ? 9 : 8)) return 1;
+    return S;
 }
 
 // Split of a thin launch (thin.cuh): `tiles` 128-row weight tiles over k_blocks
