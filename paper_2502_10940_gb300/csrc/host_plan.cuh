@@ -242,7 +242,7 @@ void set_splits(GemmParams& p, int S)
 // the K range of each tile is split (>= 4 k-blocks per split, up to about one
 // unit per SM); the fp32 partials are reduced, and the epilogue applied, by the
 // reduce kernel.  The Y GEMMs of r >= 1024 above 64 tokens, and the Z/H GEMMs of 33
-// to 64 tokens at r < 256 (but for GELU), or of any number while the cluster
+// to 48 tokens at r < 256 (64 in one tile; not GELU's), or of any number while the cluster
 // reduction (rank_gemm_splits) is switched off.  A shorter K
 // streams too little per tile for the extra reduce launch to pay off (measured:
 // the 2048-token 60M layer, K = 512 / 128, got slower).  1 = no split.
@@ -292,9 +292,10 @@ int cluster_splits(int tiles, int k_blocks, int sms, int* cost = nullptr)
 //   Z   from K = 1024 on (13 k-blocks with few tiles): shorter ones are no slower
 //       unsplit (forward of 2 to 74 tiles, split against unsplit: 8 k-blocks 1.12 to
 //       1.27, 12 1.04 to 1.21, 13 and 14 0.97 to 1.02 up to 24 tiles and 1.05 to 1.17
-//       above; from 16 on the other way is the slabs', 0.65 to 0.97), and above 64
-//       tokens: with fewer rows the slabs' reduce is the shorter way (one tile of 40
-//       tokens, K = 1024 to 11008 1.05 to 1.11, of 128 tokens 0.88 to 0.95).
+//       above; from 16 on the other way is the slabs', 0.65 to 0.97), and above 48
+//       tokens, or 64 in one tile: with fewer rows the slabs' reduce is the shorter way
+//       (one tile of 40 tokens, K = 1024 to 11008 1.05 to 1.11, of 128 tokens 0.88 to
+//       0.95; three tiles of 40 tokens 1.04, of 64 0.94 to 0.96).
 //   dZ  where the split takes enough k-blocks off the longest CTA to pay for the
 //       exchange (whole backward, split against unsplit: 5 fewer 1.00 to 1.04, 8
 //       0.93 to 1.03; in two splits, whose SMs the unsplit tiles half fill, 8 fewer
@@ -311,7 +312,7 @@ int rank_gemm_splits(int64_t n, int64_t N, int64_t K, int count, int sigma, int 
     if (2 * tiles > sms) return 1;
     const int kb = static_cast<int>((K + BK - 1) / BK);
     const bool cheap = sigma != SIG_GELU;
-    if (cheap && !dz && (n <= THIN_MAX_TOKENS || kb < 13 || (kb < 16 && tiles > 24))) return 1;
+    if (cheap && !dz && (n <= (tiles == 1 ? 64 : 48) || kb < 13 || (kb < 16 && tiles > 24))) return 1;
     const int S = cluster_splits(static_cast<int>(tiles), kb, sms);
     if (cheap && dz && n > THIN_MAX_TOKENS && kb - (kb + S - 1) / S < (S == 2 ? 9 : 8)) return 1;
     return S;
