@@ -627,13 +627,32 @@ bool fused_fwd_applies(const Shape& s, int sms)
 
 // The forward GEMMs of a few tokens run on the thin kernels (thin.cuh), except
 // the lone layers that have the single-kernel form, whose two GEMMs have to
-// match it bit for bit.  Above 32 tokens their epilogue (a token a warp at a
-// time) needs the splits that r >= 256 allows: blocks of 64 tokens, r = 256
-// 46.5 -> 45.1 us, but a gated MLP of 57 tokens, r = 128 23.7 -> 25.3 us.
+// match it bit for bit.  Above 32 tokens the epilogue (a token a warp at a time)
+// needs the splits that r >= 256 allows: blocks of 64 tokens, r = 256 46.5 -> 45.1
+// us, but a gated MLP of 57 tokens, r = 128 23.7 -> 25.3 us.
 bool thin_applies(const Shape& s, int count, int sms)
 {
     if (s.n > THIN_MAX_TOKENS || (s.n > 32 && s.r < 256)) return false;
     return !(count == 1 && fused_fwd_form(s, sms));
+}
+
+// Whether Y, and the gated product, do too.  Above 32 tokens Y has the splits for it
+// only from r = 512 on, above 48 from r = 1024; and a gated product's exchange of
+// both halves pays only with few tiles, the fewer the shorter K.  Whole forwards, thin
+// against token-major output GEMMs behind the same Z/H launch: q/k/v of 48 tokens,
+// 3008 wide, r = 320 13.0 against 10.8 us; 56 tokens, 2048, r = 512 13.8 and 12.1, r =
+// 1024 15.7 and 16.7; gated, 48 tokens, 2048 -> 5461, r = 256 12.1 and 10.2, r = 512
+// 15.3 and 13.3, r = 1024 16.6 and 17.8; 1024 -> 2736, r = 512 10.9 and 11.6; 33
+// tokens, 3008 -> 8022, r = 384 12.9 and 12.7, r = 640 14.1 and 15.5; 64 tokens, 2048
+// -> 5461, r = 1024 17.6 and 18.7, 4096 -> 11008 23.9 and 21.0.
+bool thin_y_applies(const Shape& s) { return s.n <= 32 || s.r >= (s.n <= 48 ? 512 : 1024); }
+
+bool thin_glu_applies(const Shape& s)
+{
+    if (s.n <= 32) return true;
+    const int64_t tiles = (s.d_out + BM - 1) / BM;
+    if (s.n > 48) return s.r >= 1024 && tiles <= 48;
+    return s.r >= 640 ? tiles <= 72 : s.r >= 320 && tiles <= 32;
 }
 
 // F1 of a few tokens: Z = X A^T (stored when not null), H = sigma(Z), N = r or
@@ -1213,10 +1232,11 @@ cola_status_t cola_fwd(const cola_desc_t* desc, const void* X, const void* A, co
     void* Ys[1] = {Y};
     if (thin_applies(s, 1, sms)) {
         COLA_TRY(run_thin_f1(s, desc->sigma, s.r, X, A, Z_save, H, status, sms, st));
-        return run_thin_f2(s, 1, H, s.r, Bs, Ys, status, sms, st);
+        if (thin_y_applies(s)) return run_thin_f2(s, 1, H, s.r, Bs, Ys, status, sms, st);
+    } else {
+        COLA_TRY(align_fwd_weight(*desc, &s, s.r, &A, ws, ws_bytes, L, sms, st));
+        COLA_TRY(run_f1(s, desc->sigma, s.r, X, A, Z_save, H, s.r, part, part_bytes, status, sms, st));
     }
-    COLA_TRY(align_fwd_weight(*desc, &s, s.r, &A, ws, ws_bytes, L, sms, st));
-    COLA_TRY(run_f1(s, desc->sigma, s.r, X, A, Z_save, H, s.r, part, part_bytes, status, sms, st));
     return run_f2(s, 1, Hs, s.r, Bs, Ys, part, part_bytes, status, sms, st);
 }
 
@@ -1323,10 +1343,11 @@ cola_status_t cola_fwd_gate_up(const cola_desc_t* desc, const void* X, const voi
     const size_t part_bytes = L.total - L.part_off;
     if (thin_applies(s, 2, sms)) {
         COLA_TRY(run_thin_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, status, sms, st));
-        return run_thin_glu(s, H, B_gate, B_up, M, Y_gate, Y_up, status, sms, st);
+        if (thin_glu_applies(s)) return run_thin_glu(s, H, B_gate, B_up, M, Y_gate, Y_up, status, sms, st);
+    } else {
+        COLA_TRY(align_fwd_weight(*desc, &s, R, &A_cat, ws, ws_bytes, L, sms, st));
+        COLA_TRY(run_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, R, part, part_bytes, status, sms, st));
     }
-    COLA_TRY(align_fwd_weight(*desc, &s, R, &A_cat, ws, ws_bytes, L, sms, st));
-    COLA_TRY(run_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, R, part, part_bytes, status, sms, st));
     return run_glu(s, H, R, B_gate, B_up, M, Y_gate, Y_up, status, sms, st);
 }
 
@@ -1353,10 +1374,11 @@ cola_status_t cola_fwd_shared_x(const cola_desc_t* desc, int32_t count, const vo
     const size_t part_bytes = L.total - L.part_off;
     if (thin_applies(s, count, sms)) {
         COLA_TRY(run_thin_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, status, sms, st));
-        return run_thin_f2(s, count, H, R, B, Y, status, sms, st);
+        if (thin_y_applies(s)) return run_thin_f2(s, count, H, R, B, Y, status, sms, st);
+    } else {
+        COLA_TRY(align_fwd_weight(*desc, &s, R, &A_cat, ws, ws_bytes, L, sms, st));
+        COLA_TRY(run_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, R, part, part_bytes, status, sms, st));
     }
-    COLA_TRY(align_fwd_weight(*desc, &s, R, &A_cat, ws, ws_bytes, L, sms, st));
-    COLA_TRY(run_f1(s, desc->sigma, R, X, A_cat, Z_cat, H, R, part, part_bytes, status, sms, st));
     const void* Hs[3] = {H, H + slice, H + 2 * slice};
     return run_f2(s, count, Hs, R, B, Y, part, part_bytes, status, sms, st);
 }
@@ -1446,7 +1468,7 @@ cola_status_t cola_recompute_up(const cola_desc_t* desc, int32_t count, const vo
     COLA_TRY(launched(traced(COLA_KERNEL_SIGMA, 1, mnk, 1, 0, st, [&] {
         return launch_sigma(Z_cat, H, static_cast<long long>(s.n) * R, desc->sigma, sms, st);
     })));
-    if (thin_applies(s, count, sms)) return run_thin_f2(s, count, H, R, B, Y, status, sms, st);
+    if (thin_applies(s, count, sms) && thin_y_applies(s)) return run_thin_f2(s, count, H, R, B, Y, status, sms, st);
     const size_t slice = static_cast<size_t>(s.r) * 2;
     const void* Hs[3] = {H, H + slice, H + 2 * slice};
     float* part = reinterpret_cast<float*>(wsb(ws) + L.part_off);

@@ -323,13 +323,22 @@ int rank_gemm_splits(int64_t n, int64_t N, int64_t K, int count, int sigma, int 
 // k-blocks each, 1.6 CTAs per SM at most (measured, 7B-shaped block of one
 // token: 61.3 us at 1.25, 58.6 at 1.6, 64.4 at 2; 1B-shaped, 32 tokens: 45.1,
 // 44.0, 44.9); the operand ring as deep as lets two CTAs, or one and a CTA of
-// the kernel before, share an SM.
-void thin_splits(ThinBatch& b, bool glu, int sms)
+// the kernel before, share an SM.  A gated product of more than 48 tokens in
+// splits takes more shared memory than that, so its splits are counted for one CTA
+// per SM: 43 tiles of 57 tokens, r = 512 21.1 us a call for 1.6 and 14.8 for one.
+// The SMs of a cluster lie in one partition of the GPU, so it runs at most 14
+// clusters of more than 13 CTAs at once, two a partition, and three of 13: Z of 16
+// tokens, 15 tiles of 86 k-blocks 14.8 us in fifteens and 9.3 for 14 tiles, 17 tiles
+// in thirteens 10.0.
+constexpr int THIN_WIDE_CLUSTER = 13, THIN_WIDE_CLUSTERS = 14;
+
+void thin_splits(ThinBatch& b, bool glu, int sms, bool one_per_sm = false)
 {
     b.NT = (b.n + 15) / 16 * 16;
-    int s = sms * 8 / 5 / b.tiles;
+    int s = (one_per_sm ? sms : sms * 8 / 5) / b.tiles;
     if (s > (b.k_blocks + 1) / 2) s = (b.k_blocks + 1) / 2;
     if (s > THIN_MAX_CLUSTER) s = THIN_MAX_CLUSTER;
+    if (s > THIN_WIDE_CLUSTER && b.tiles > THIN_WIDE_CLUSTERS) s = THIN_WIDE_CLUSTER;
     if (s < 1) s = 1;
     b.kps = (b.k_blocks + s - 1) / s;
     b.S = (b.k_blocks + b.kps - 1) / b.kps;   // no empty split
@@ -340,6 +349,7 @@ void thin_splits(ThinBatch& b, bool glu, int sms)
     if (b.stages > iters) b.stages = iters;
     if (b.stages > THIN_MAX_STAGES) b.stages = THIN_MAX_STAGES;
     if (b.stages < 2) b.stages = 2;
+    if (!one_per_sm && thin_smem_bytes(b.stages, b.NT, b.S, b.TB, glu) > THIN_SMEM_BUDGET) thin_splits(b, glu, sms, true);
 }
 
 int64_t partial_elems(const GemmParams& p, int bn, int msub)
