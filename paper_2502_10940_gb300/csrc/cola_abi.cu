@@ -139,23 +139,8 @@ WgradPlan wgrad_plan(const cola_desc_t& d, int nproj, int sms)
     }
     M[nb] = R;
     N[nb] = d.d_in;
-    return plan_wgrad(M, N, nb + 1, d.n, sms);
+    return plan_wgrad(M, N, nb + 1, d.n, d.wgrad_fp32 != 0, sms);
 }
-
-// The split-tail schedule of the same group (bf16 gradients): the tile
-// configuration of wgrad_plan.  It runs when its cost is no higher than the
-// uniform token split's (tail_wins).
-TailPlan wgrad_tail_plan(const WgradPlan& w, int64_t ntok, int sms)
-{
-    GemmParams p[MAX_GROUP];
-    for (int j = 0; j < w.count; ++j) {
-        p[j] = base_params(w.p[j].M, w.p[j].N, ntok, w.bn, w.msub);
-        p[j].n_major = w.p[j].n_major;
-    }
-    return plan_tail(p, w.count, w.bn, w.msub, sms);
-}
-
-bool tail_wins(const WgradPlan& w, const TailPlan& t) { return t.cost <= w.cost; }
 
 // fp32 partial elements the forward of `nproj` projections needs when its
 // GEMMs are small enough to be split over K into slabs (small_launch_splits),
@@ -164,7 +149,7 @@ int64_t fwd_part_elems(const cola_desc_t& d, int nproj, int sms)
 {
     int64_t need = 0;
     const int64_t R = nproj * d.r;
-    const int bn1 = fill_bn(d.n, R, d.d_in, 1, sms);
+    const int bn1 = fill_bn(d.n, R, d.d_in, 1, sms, PAD_K_SIGMA);
     if (choose_msub(d.n, R, d.d_in, bn1) == 1) {
         GemmParams p = base_params(d.n, R, d.d_in, bn1, 1);
         const int S = small_launch_splits(p.m_tiles * p.n_tiles, p.k_blocks, sms);
@@ -173,7 +158,7 @@ int64_t fwd_part_elems(const cola_desc_t& d, int nproj, int sms)
             need = std::max<int64_t>(need, p.splits * partial_elems(p, bn1, 1));
         }
     }
-    const int bn2 = fill_bn(d.n, d.d_out, d.r, nproj, sms);
+    const int bn2 = fill_bn(d.n, d.d_out, d.r, nproj, sms, PAD_K_STORE);
     if (choose_msub(d.n, d.d_out, d.r, bn2) == 1) {
         GemmParams p = base_params(d.n, d.d_out, d.r, bn2, 1);
         const int S = small_launch_splits(nproj * p.m_tiles * p.n_tiles, p.k_blocks, sms);
@@ -470,9 +455,10 @@ bool fused_bwd_form(const Shape& s, int sms);
 // 30000 (4) the same; backward 202 -> 196, 92.2 -> 89.9, 120.1 -> 120.5, the same.
 struct AlignRule {
     double pair_flops, single_flops;
+    int64_t pad_k;   // of the GEMM's column tile (fill_bn)
 };
-constexpr AlignRule ALIGN_FWD{24e9, 8e9};
-constexpr AlignRule ALIGN_DX{60e9, 12e9};
+constexpr AlignRule ALIGN_FWD{24e9, 8e9, PAD_K_SIGMA};
+constexpr AlignRule ALIGN_DX{60e9, 12e9, PAD_K_STORE};
 constexpr int64_t ALIGN_SINGLE_TOKENS = 8192;
 
 cola_status_t align_weight(Shape* s, int64_t R, const void** A, int64_t K, int64_t N, const AlignRule& rule,
@@ -480,7 +466,7 @@ cola_status_t align_weight(Shape* s, int64_t R, const void** A, int64_t K, int64
 {
     const int64_t ld = (s->d_in + 63) / 64 * 64;
     if (s->ld_a % 16 == 0) return COLA_OK;
-    const bool pair = choose_msub(s->n, N, K, choose_bn_for(s->n, N, K)) == TILE_PAIR;
+    const bool pair = choose_msub(s->n, N, K, fill_bn(s->n, N, K, 1, sms, rule.pad_k)) == TILE_PAIR;
     if (2.0 * s->n * N * K < (pair ? rule.pair_flops : rule.single_flops)) return COLA_OK;
     if (!pair && s->n < ALIGN_SINGLE_TOKENS) return COLA_OK;
     if (static_cast<size_t>(R) * ld * 2 > room_bytes) return COLA_OK;
@@ -539,7 +525,7 @@ cola_status_t run_f1(const Shape& s, int sigma, int64_t N, const void* X, const 
         g.ldo = ldz;
         return run_cluster_rank(CRED_ZH, sigma, 1, s.n, N, s.d_in, g, Sc, status, st);
     }
-    const int bn = fill_bn(s.n, N, s.d_in, 1, sms);
+    const int bn = fill_bn(s.n, N, s.d_in, 1, sms, PAD_K_SIGMA);
     const int ms = choose_msub(s.n, N, s.d_in, bn);
     GemmProblem pr;
     std::memset(&pr, 0, sizeof pr);
@@ -845,7 +831,7 @@ cola_status_t run_fused_bwd(const Shape& s, int sigma, const void* dY, const voi
 cola_status_t run_f2(const Shape& s, int count, const void* const* H, int64_t ldh, const void* const* B,
                      void* const* Y, float* part, size_t part_bytes, unsigned int* status, int sms, cudaStream_t st)
 {
-    const int bn = fill_bn(s.n, s.d_out, s.r, count, sms);
+    const int bn = fill_bn(s.n, s.d_out, s.r, count, sms, PAD_K_STORE);
     const int ms = choose_msub(s.n, s.d_out, s.r, bn);
     GemmProblem pr[MAX_GROUP];
     int64_t mnk[MAX_GROUP][3];
@@ -935,7 +921,7 @@ cola_status_t run_b1(const Shape& s, int sigma, int count, const void* const* dY
         }
         return run_cluster_rank(CRED_DZ, sigma, count, s.n, s.r, s.d_out, g, Sc, status, st);
     }
-    const int bn = fill_bn(s.n, s.r, s.d_out, count, sms);
+    const int bn = fill_bn(s.n, s.r, s.d_out, count, sms, PAD_K_SIGMA);
     const int ms = choose_msub(s.n, s.r, s.d_out, bn);
     GemmProblem pr[MAX_GROUP];
     int64_t mnk[MAX_GROUP][3];
@@ -1164,7 +1150,7 @@ cola_status_t run_b4_glu(const Shape& s, int64_t K, const void* dZ, int64_t ldz,
 cola_status_t run_b4(const Shape& s, int64_t K, const void* dZ, int64_t ldz, const void* A, void* dX,
                      unsigned int* status, int sms, cudaStream_t st)
 {
-    const int bn = fill_bn(s.n, s.d_in, K, 1, sms);
+    const int bn = fill_bn(s.n, s.d_in, K, 1, sms, PAD_K_STORE);
     const int ms = choose_msub(s.n, s.d_in, K, bn);
     const bool wide = store_boxes64(ms == TILE_PAIR, s.d_in, s.ld_x);
     GemmProblem pr;

@@ -88,10 +88,10 @@ bool map_mnmajor(CUtensorMap* m, const void* base, int64_t mn_extent, int64_t k_
 // ------------------------------------------------------------ planning
 // Column tile: the width that pads N least; a compute-heavy GEMM with K >= 512
 // (`pairs`) takes 256, because only 256-column tiles run on CTA pairs, which
-// outweighs the padding (at most a third of the tile columns).  Measured against
-// 128-column tiles wherever 256 pads N by more than 5 % (forward + backward):
-// 16384 tokens 2600 -> 2600, r = 640 396 -> 301 us; 12000, 3300 -> 3300, r = 832
-// 427 -> 357; 65536, 1500 -> 1500, r = 384 479 -> 439.
+// outweighs the padding where fill_bn leaves it.  Measured against 128-column tiles
+// wherever 256 pads N by more than 5 % (forward + backward): 16384 tokens 2600 ->
+// 2600, r = 640 396 -> 301 us; 12000, 3300 -> 3300, r = 832 427 -> 357; 65536, 1500 ->
+// 1500, r = 384 479 -> 439; 67708, 1536 -> 1536, r = 320 446 -> 409.
 int choose_bn(int64_t N, bool pairs = false)
 {
     if (N <= 128) return 128;
@@ -134,13 +134,41 @@ int choose_bn_for(int64_t M, int64_t N, int64_t K)
     return choose_bn(N, heavy_gemm(M, N, K) && K >= 512);
 }
 
-// The same for `count` GEMMs of one launch, with 128 columns where those tiles
-// still run in one wave: twice the CTAs of 256-column ones.
-int fill_bn(int64_t M, int64_t N, int64_t K, int count, int sms)
+// Whether 256-column tiles round N up further than 128-column ones do, and by more
+// than the 5 % that CTA pairs always outweigh from N = 1024 on.
+bool pairs_pad(int64_t N)
+{
+    const int64_t pad256 = (N + 255) / 256 * 256;
+    return pad256 > (N + 127) / 128 * 128 && !(N >= 1024 && pad256 * 100 <= N * 105);
+}
+
+// Where a GEMM that pairs would pad starts taking them.
+// The epilogues of Z and dZ outlast the MMAs of a shorter walk, and a pair's two CTAs
+// then wait for them together: pairs against 128-column tiles, K = 512, r = 384, 832
+// Z 107 / 87 and 97 / 86 us, dZ 158 / 111 and 143 / 112; K = 768 Z 85 / 82, 78 / 76, dZ
+// 115 / 87, 107 / 82; K = 1024 r = 832 66 / 73 and 84 / 76.  Y and dX free their
+// accumulators before they store: K = 512 to 1024 0.85 to 1.02.
+constexpr int64_t PAD_K_SIGMA = 1024, PAD_K_STORE = 512;
+
+// The column tile of `count` GEMMs of one launch: 128 columns instead of 256
+//   - where those tiles still run in one wave (twice the CTAs of 256-column ones);
+//   - for compute-heavy GEMMs that pairs would pad, below K = pad_k, and where the
+//     padding costs more waves than pairs make up for.  A wave of pair tiles (256 x
+//     256 on two SMs) and one of two 128-row sub-tiles (256 x 128 on one) hold the same
+//     work per SM, and the first is some 20 % faster: us of Z, waves of pairs and of
+//     128-column tiles: 12715 x 384, K = 2048 (2, 1) 36.9 / 29.2; 10926 x 832, 1100 (3, 2)
+//     35.7 / 31.8; 50781 x 320, 2048 (6, 4) 81.4 / 75.4; 26702 x 640, 2048 (5, 4) 67.5 /
+//     71.0; 16954 x 384, 3072 (2, 2) 47.7 / 58.0.
+int fill_bn(int64_t M, int64_t N, int64_t K, int count, int sms, int64_t pad_k)
 {
     const int bn = choose_bn_for(M, N, K);
-    if (bn == 128 || heavy_gemm(M, N, K)) return bn;
-    return count * ((M + BM - 1) / BM) * ((N + 127) / 128) <= sms ? 128 : 256;
+    if (bn == 128) return bn;
+    const int64_t n256 = (N + 255) / 256, n128 = (N + 127) / 128;
+    if (!heavy_gemm(M, N, K)) return count * ((M + BM - 1) / BM) * n128 <= sms ? 128 : 256;
+    if (!pairs_pad(N)) return bn;
+    const int64_t units = count * ((M + 2 * BM - 1) / (2 * BM)), pairs = sms / 2;
+    const int64_t waves256 = (units * n256 + pairs - 1) / pairs, waves128 = (units * n128 + sms - 1) / sms;
+    return K < pad_k || 4 * waves256 > 5 * waves128 ? 128 : bn;
 }
 
 // Whether plain outputs of N columns and pitch `ld` are stored through 64-column
@@ -402,42 +430,6 @@ WgradPlan plan_wgrad_tiles(const int64_t* M, const int64_t* N, int count, int64_
     return w;
 }
 
-WgradPlan plan_wgrad(const int64_t* M, const int64_t* N, int count, int64_t ntok, int sms)
-{
-    int bn = 256;
-    for (int i = 0; i < count; ++i) {
-        const int b = choose_bn_for(M[i], N[i], ntok);
-        bn = b < bn ? b : bn;
-    }
-    int msub = TILE_PAIR;   // the smallest tile any GEMM of the group would take
-    for (int i = 0; i < count; ++i) {
-        const int ms = choose_msub(M[i], N[i], ntok, bn);
-        if (ms == 1 || (ms == 2 && msub == TILE_PAIR)) msub = ms;
-    }
-    if (bn == 256 && msub == 1) {   // 128 columns where those tiles still run in one wave
-        int64_t t = 0;
-        for (int i = 0; i < count; ++i) t += ((M[i] + BM - 1) / BM) * ((N[i] + 127) / 128);
-        if (t <= sms) bn = 128;
-    }
-    return plan_wgrad_tiles(M, N, count, ntok, bn, msub, sms);
-}
-
-// The plan of one gradient whose partial tile grid has to fit `limit` bytes even
-// unsplit, with the token split reduced until its slabs do.  Wide tiles round M and
-// N up further: when their grid is too large, 128-column tiles, and then 128 x 128
-// ones, whose grid is the smallest.  false: not even that fits.
-bool plan_wgrad_within(int64_t M, int64_t N, int64_t ntok, size_t limit, int sms, WgradPlan* w)
-{
-    const auto slab = [&] { return static_cast<size_t>(w->slab[0]) * 4; };
-    *w = plan_wgrad(&M, &N, 1, ntok, sms);
-    if (slab() > limit) *w = plan_wgrad_tiles(&M, &N, 1, ntok, 128, choose_msub(M, N, ntok, 128), sms);
-    if (slab() > limit) *w = plan_wgrad_tiles(&M, &N, 1, ntok, 128, 1, sms);
-    if (slab() > limit) return false;
-    const int max_splits = static_cast<int>(limit / slab());
-    if (w->p[0].splits > max_splits) set_splits(w->p[0], max_splits);
-    return true;
-}
-
 // Split-tail schedule of a weight-gradient launch with bf16 outputs
 // (EPI_TAIL).  The output tiles run whole in waves of `slots` CTAs (CTA
 // pairs); the CTAs of a wave walk the token range in step, so the operand
@@ -513,6 +505,82 @@ TailPlan plan_tail(const GemmParams* p, int count, int bn, int msub, int sms)
         }
     }
     return s;
+}
+
+// The split-tail schedule of a planned group (bf16 gradients), with its tiles.  It runs
+// when its cost is no higher than the uniform token split's (tail_wins).
+TailPlan wgrad_tail_plan(const WgradPlan& w, int64_t ntok, int sms)
+{
+    GemmParams p[MAX_GROUP];
+    for (int j = 0; j < w.count; ++j) {
+        p[j] = base_params(w.p[j].M, w.p[j].N, ntok, w.bn, w.msub);
+        p[j].n_major = w.p[j].n_major;
+    }
+    return plan_tail(p, w.count, w.bn, w.msub, sms);
+}
+
+bool tail_wins(const WgradPlan& w, const TailPlan& t) { return t.cost <= w.cost; }
+
+// k-block steps of a planned group by the schedule it runs (`uniform`: fp32 gradients
+// never take the split tail), for comparing tile sizes: a tail's few tiles are reduced
+// in about half of REDUCE_LAUNCH_KB.
+double wgrad_cost(const WgradPlan& w, int64_t ntok, bool uniform, int sms)
+{
+    if (uniform) return w.cost;
+    const TailPlan t = wgrad_tail_plan(w, ntok, sms);
+    return tail_wins(w, t) ? t.cost - (t.pieces > 1 ? 0.5 * REDUCE_LAUNCH_KB : 0.0) : w.cost;
+}
+
+// The plan of a group with the widest tiles all its GEMMs would take.  CTA pairs that pad
+// a width (by more than fill_bn lets pass) run it where their schedule takes no more
+// than 5/4 of the steps of 128-column tiles, which are of equal work per SM and some 20 %
+// slower; steps, pairs and 128 columns, and us with the reduce: 16276 tokens 2560 -> 2560,
+// r = 384 (199, 151) 83.7 / 72.0; 8877, 1100 -> 1100, r = 1024 (130, 93) 57.1 / 50.5; 25431,
+// 2560 -> 2560, r = 384 (284, 222) 112.5 / 100.3; 14305, 5461 -> 5461, r = 384 (280, 224)
+// 102.6 / 104.3; 23475, 1024 -> 1024, r = 832 (205, 179) 83.8 / 85.9.
+WgradPlan plan_wgrad(const int64_t* M, const int64_t* N, int count, int64_t ntok, bool uniform, int sms)
+{
+    int bn = 256;
+    for (int i = 0; i < count; ++i) {
+        const int b = choose_bn_for(M[i], N[i], ntok);
+        bn = b < bn ? b : bn;
+    }
+    const auto tile_mode = [&](int cols) {   // the smallest tile any GEMM of the group would take
+        int msub = TILE_PAIR;
+        for (int i = 0; i < count; ++i) {
+            const int ms = choose_msub(M[i], N[i], ntok, cols);
+            if (ms == 1 || (ms == 2 && msub == TILE_PAIR)) msub = ms;
+        }
+        return msub;
+    };
+    const int msub = tile_mode(bn);
+    if (bn == 256 && msub == 1) {   // 128 columns where those tiles still run in one wave
+        int64_t t = 0;
+        for (int i = 0; i < count; ++i) t += ((M[i] + BM - 1) / BM) * ((N[i] + 127) / 128);
+        if (t <= sms) bn = 128;
+    }
+    const WgradPlan w = plan_wgrad_tiles(M, N, count, ntok, bn, msub, sms);
+    bool padded = false;
+    for (int i = 0; i < count; ++i) padded = padded || pairs_pad(N[i]);
+    if (msub != TILE_PAIR || !padded) return w;
+    const WgradPlan narrow = plan_wgrad_tiles(M, N, count, ntok, 128, tile_mode(128), sms);
+    return wgrad_cost(w, ntok, uniform, sms) > 1.25 * wgrad_cost(narrow, ntok, uniform, sms) ? narrow : w;
+}
+
+// The plan of one gradient whose partial tile grid has to fit `limit` bytes even
+// unsplit, with the token split reduced until its slabs do.  Wide tiles round M and
+// N up further: when their grid is too large, 128-column tiles, and then 128 x 128
+// ones, whose grid is the smallest.  false: not even that fits.
+bool plan_wgrad_within(int64_t M, int64_t N, int64_t ntok, size_t limit, int sms, WgradPlan* w)
+{
+    const auto slab = [&] { return static_cast<size_t>(w->slab[0]) * 4; };
+    *w = plan_wgrad(&M, &N, 1, ntok, true, sms);
+    if (slab() > limit) *w = plan_wgrad_tiles(&M, &N, 1, ntok, 128, choose_msub(M, N, ntok, 128), sms);
+    if (slab() > limit) *w = plan_wgrad_tiles(&M, &N, 1, ntok, 128, 1, sms);
+    if (slab() > limit) return false;
+    const int max_splits = static_cast<int>(limit / slab());
+    if (w->p[0].splits > max_splits) set_splits(w->p[0], max_splits);
+    return true;
 }
 
 // The tile configuration dispatch() launches for a planned (bn, msub): bit 2
