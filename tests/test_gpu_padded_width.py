@@ -64,3 +64,21 @@ def test_tiles_of_padded_widths(n, d_in, d_out, r, zh, y, dz, dx, wgrad):
     assert _rel(dB, f(dY).T @ f(H)) < 5e-3
     for t in (Y, dX):
         assert torch.as_strided(t, (n, t.stride(0)), (t.stride(0), 1))[:, t.shape[1]:].isnan().all()
+
+
+# 128-column tiles would run unsplit in one wave (71 k-block steps), 256-column ones split three ways take 47
+def test_weight_gradients_split_where_wide_tiles_take_far_fewer_steps():
+    from paper_2502_10940_gb300 import cola
+    n, d_in, d_out, r = 4500, 456, 4584, 192
+    X, dY = I.normal_bf16(n, d_in, 1.0, 1, "cuda"), I.normal_bf16(n, d_out, 1.0, 2, "cuda")
+    A, B = I.normal_bf16(r, d_in, d_in ** -0.5, 3, "cuda"), I.normal_bf16(d_out, r, r ** -0.5, 4, "cuda")
+    Z, H = I.normal_bf16(n, r, 1.0, 5, "cuda"), I.normal_bf16(n, r, 1.0, 6, "cuda")
+    d = cola.desc(n, d_in, d_out, r, sigma="identity", mode="cola")
+    ws = cola.workspace(d)
+    dX, dA, dB = torch.empty_like(X), torch.empty_like(A), torch.empty_like(B)
+    with cola.Trace(16) as tr:
+        cola.cola_bwd(d, X, A, B, dY, Z, H, dX, dA, dB, ws)
+    assert [t[2] for t in tr.records() if t[0] == "wgrad"] == [3], tr.records()
+    f = torch.Tensor.float
+    assert _rel(dB, f(dY).T @ f(H)) < 3e-3                     # one bf16 rounding
+    assert _rel(dA, (f(dY) @ f(B)).T @ f(X)) < 5e-3            # and dZ's
