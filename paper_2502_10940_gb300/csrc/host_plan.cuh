@@ -320,9 +320,9 @@ int cluster_splits(int tiles, int k_blocks, int sms, int* cost = nullptr)
 //   Z   from K = 1024 on (13 k-blocks with few tiles): shorter ones are no slower
 //       unsplit (forward of 2 to 74 tiles, split against unsplit: 8 k-blocks 1.12 to
 //       1.27, 12 1.04 to 1.21, 13 and 14 0.97 to 1.02 up to 24 tiles and 1.05 to 1.17
-//       above; from 16 on the other way is the slabs', 0.65 to 0.97), and above 48
-//       tokens, or 64 in one tile: with fewer rows the slabs' reduce is the shorter way
-//       (one tile of 40 tokens, K = 1024 to 11008 1.05 to 1.11, of 128 tokens 0.88 to
+//       above; from 16 on the other way is the slabs', 0.65 to 0.97, and above 48
+//       tokens, or 64 in one tile: with fewer rows their reduce is the shorter way: one
+//       tile of 40 tokens, K = 1024 to 11008 1.05 to 1.11, of 128 tokens 0.88 to
 //       0.95; three tiles of 40 tokens 1.04, of 64 0.94 to 0.96).
 //   dZ  where the split takes enough k-blocks off the longest CTA to pay for the
 //       exchange (whole backward, split against unsplit: 5 fewer 1.00 to 1.04, 8
@@ -332,7 +332,9 @@ int cluster_splits(int tiles, int k_blocks, int sms, int* cost = nullptr)
 // Both hold for SiLU and the identity.  GELU's elementwise work outweighs the
 // exchange, and the splits share it out: split for every K that can be (gated MLP
 // of 783 tokens, 960 -> 2176, r = 192 15.9 -> 14.0 us, 585 tokens, 696 -> 1536, r =
-// 128, two projections 14.9 -> 12.7; 52 tokens, 862 -> 2304 14.0 -> 9.8).
+// 128, two projections 14.9 -> 12.7; 52 tokens, 862 -> 2304 14.0 -> 9.8), but for a dZ
+// of many tiles and few k-blocks (us, unsplit and split, 56 tiles of 9 13.4, 15.9; a
+// backward with 76 of 13 51.8, 49.6, with 54 of 16 42.6, 39.8).
 int rank_gemm_splits(int64_t n, int64_t N, int64_t K, int count, int sigma, int sms, bool dz)
 {
     if (heavy_gemm(n, N, K)) return 1;
@@ -340,9 +342,10 @@ int rank_gemm_splits(int64_t n, int64_t N, int64_t K, int count, int sigma, int 
     if (2 * tiles > sms) return 1;
     const int kb = static_cast<int>((K + BK - 1) / BK);
     const bool cheap = sigma != SIG_GELU;
-    if (cheap && !dz && (n <= (tiles == 1 ? 64 : 48) || kb < 13 || (kb < 16 && tiles > 24))) return 1;
+    if (cheap && !dz && (kb < 16 ? kb < 13 || tiles > 24 : n <= (tiles == 1 ? 64 : 48))) return 1;
     const int S = cluster_splits(static_cast<int>(tiles), kb, sms);
-    if (cheap && dz && n > THIN_MAX_TOKENS && kb - (kb + S - 1) / S < (S == 2 ? 9 : 8)) return 1;
+    const int least = cheap ? (S == 2 ? 9 : 8) : (tiles >= 48 ? 5 : 0);   // k-blocks saved
+    if (dz && n > THIN_MAX_TOKENS && kb - (kb + S - 1) / S < least) return 1;
     return S;
 }
 
