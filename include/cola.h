@@ -315,6 +315,19 @@ cola_status_t cola_selftest_wait_timeout_pair(void* ws, size_t ws_bytes, int32_t
  * usable.  Async on `stream`. */
 cola_status_t cola_selftest_wait_timeout_cluster(void* ws, size_t ws_bytes, void* stream);
 
+/* The same self-test on the kernel of the forward GEMMs of a few tokens: Y of
+ * two tokens, a 128 x 384 weight, on a cluster of three CTAs that split K and
+ * own a token, a token and none.  In ws after its status header lie the weight,
+ * the tokens [2 x 384] and Y [2 x 128] (ws_bytes >= 256 + 98 KB).  CTA 1
+ * issues no loads: its MMA issuer gives up after 2 s, and it still sends its
+ * (zero) partial bands so that CTA 0 completes and stores token 0 of Y; CTA 1
+ * stores nothing.  The next cola_check_status on ws returns
+ * COLA_ERR_DEVICE_TIMEOUT with some of COLA_STATUS_PRODUCER_TIMEOUT,
+ * COLA_STATUS_MMA_TIMEOUT and COLA_STATUS_EPILOGUE_TIMEOUT set and not
+ * COLA_STATUS_DRAIN_TIMEOUT (the exchange of the three CTAs completed), and the
+ * CUDA context stays usable.  Async on `stream`. */
+cola_status_t cola_selftest_wait_timeout_thin(void* ws, size_t ws_bytes, void* stream);
+
 /* ---- weight gradient without any workspace or allocation ----
  * The paper has no counterpart to this entry point.  It serves callers that
  * cannot allocate device memory: an operator or plugin interface that hands

@@ -1553,6 +1553,38 @@ cola_status_t cola_selftest_wait_timeout_cluster(void* ws, size_t ws_bytes, void
                            }));
 }
 
+cola_status_t cola_selftest_wait_timeout_thin(void* ws, size_t ws_bytes, void* stream)
+{
+    if (!ws) return COLA_ERR_INVALID;
+    if (reinterpret_cast<uintptr_t>(ws) & (WS_ALIGN - 1)) return COLA_ERR_ALIGN;
+    constexpr int64_t M = 128, K = 384, n = 2;   // one weight tile, 6 k-blocks, 2 tokens
+    constexpr size_t w_bytes = M * K * 2, t_bytes = n * K * 2, y_bytes = n * M * 2;
+    if (ws_bytes < WS_HEADER + w_bytes + t_bytes + y_bytes) return COLA_ERR_WORKSPACE;
+    uint8_t* base = wsb(ws) + WS_HEADER;
+    ThinBatch b;
+    std::memset(&b, 0, sizeof b);
+    b.count = 1;
+    b.tiles = 1;
+    b.n = static_cast<int>(n);
+    b.NT = 16;
+    b.k_blocks = static_cast<int>(K / BK);
+    b.S = 3;       // two CTAs own a token each, the third none
+    b.kps = 2;
+    b.TB = 1;
+    b.stages = 2;
+    b.status = ws_status(ws);
+    b.selftest = 1;
+    ThinProblem& P = b.prob[0];
+    COLA_MAP(map_kmajor(&P.map_w, base, K, M, K, BM));
+    COLA_MAP(map_kmajor(&b.map_t, base + w_bytes, K, n, K, b.NT));
+    P.M = static_cast<int>(M);
+    P.o0 = reinterpret_cast<__nv_bfloat16*>(base + w_bytes + t_bytes);
+    P.ldo = M;
+    const int64_t mnk[1][3] = {{n, M, K}};
+    return launched(traced(COLA_KERNEL_FWD_Y, 1, mnk, b.S, TRACE_CLUSTER, static_cast<cudaStream_t>(stream),
+                           [&] { return launch_thin(b, THIN_STORE, SIG_IDENTITY, static_cast<cudaStream_t>(stream)); }));
+}
+
 cola_status_t cola_check_status(void* ws, void* stream, uint32_t* code_out)
 {
     if (!ws) return COLA_ERR_INVALID;

@@ -76,6 +76,10 @@ struct ThinBatch {
     int stages;           // operand ring
     int early_weights;    // 1: load weights before the wait for the preceding kernel
     unsigned int* status;
+    // failure-detection self-test: 1 = CTA rank 1 of the first cluster issues
+    // no loads, so its MMA issuer's first wait runs out while the other CTAs
+    // of the cluster complete normally
+    int selftest;
 };
 
 // Dynamic shared memory: the ring (16 KB of W and NT tokens per k-block),
@@ -244,7 +248,8 @@ __global__ void __launch_bounds__(THIN_THREADS) thin_kernel(const __grid_constan
         // ------------------------------------------------ TMA producer
         if (lane == 0) {
             int issued = 0;
-            for (int i = 0; i < iters; ++i) {
+            const bool no_loads = b.selftest == 1 && tile == 0 && rank == 1;
+            for (int i = 0; i < iters && !no_loads; ++i) {
                 const int s = i % stages;
                 if (i >= stages &&
                     !wait_bounded(&empty_bar[s], static_cast<uint32_t>((i / stages) - 1) & 1u, wc, ST_TIMEOUT_PRODUCER))

@@ -8,7 +8,8 @@ CTA's loads of later stages land, in which case the pair's abort drain must
 see every load of both CTAs land (no drain-timeout bit) before it exits.  And
 on a cluster-reduced weight gradient, where one CTA of the cluster gives up on
 its main loop: it still sends its (zero) partial band, the other CTA
-completes, and the exchange between them ends without a drain timeout."""
+completes, and the exchange between them ends without a drain timeout.  The
+same on the kernel of a few tokens, with a CTA that owns no tokens."""
 import time
 
 import pytest
@@ -139,6 +140,39 @@ def test_cluster_wait_runs_out_and_exchange_completes():
     with cola.Trace(16) as tr:
         g = gpu_layer(inp, "silu", "cola")
     assert any(rec[0] == "wgrad" and rec[3] & CLUSTER for rec in tr.records()), tr.records()
+    o = oracle_layer(inp, "silu", "cola")
+    for k in ["Y", "dX", "dA", "dB"]:
+        assert_close(k, to64(g[k]), o[k])
+
+
+def test_thin_wait_runs_out_and_exchange_completes():
+    from paper_2502_10940_gb300 import cola
+    w, t, y = 128 * 384 * 2, 2 * 384 * 2, 2 * 128 * 2
+    ws = torch.zeros(256 + w + t + y, dtype=torch.uint8, device="cuda")
+    Y = ws[256 + w + t:].view(torch.bfloat16).view(2, 128)
+    Y.fill_(7.0)
+    cola.cola_workspace_init(ws)
+    assert cola.cola_check_status(ws)[0] == 0
+    t0 = time.perf_counter()
+    with cola.Trace(4) as tr:
+        cola.cola_selftest_wait_timeout_thin(ws)
+    st, code = cola.cola_check_status(ws)
+    dt = time.perf_counter() - t0
+    recs = tr.records()
+    assert len(recs) == 1 and recs[0][3] & CLUSTER and recs[0][2] == 3, recs
+    assert st == 6  # COLA_ERR_DEVICE_TIMEOUT
+    assert code & (PRODUCER | MMA | EPILOGUE), hex(code)
+    assert not code & ~(PRODUCER | MMA | EPILOGUE), hex(code)   # the exchange completed: no drain timeout
+    assert 1.5 < dt < 30.0
+    assert cola.cola_check_status(ws)[0] == 0
+    # CTA 0 stored its token, CTA 1, which gave up, not its own; the operands are as they were
+    assert bool((Y[0] == 0).all()) and bool((Y[1] == 7).all())
+    assert int(ws[256:256 + w + t].count_nonzero()) == 0
+    # the context still runs the kernel correctly
+    inp = make_inputs(5, 520, 600, 192, seed=29)
+    with cola.Trace(16) as tr:
+        g = gpu_layer(inp, "silu", "cola")
+    assert [rec[0] for rec in tr.records()][:2] == ["fwd_zh", "fwd_y"] and all(rec[3] & CLUSTER for rec in tr.records()[:2])
     o = oracle_layer(inp, "silu", "cola")
     for k in ["Y", "dX", "dA", "dB"]:
         assert_close(k, to64(g[k]), o[k])
