@@ -317,13 +317,14 @@ int cluster_splits(int tiles, int k_blocks, int sms, int* cost = nullptr)
 // q/k/v of 509 tokens, d = 1024, r = 256 23.9 -> 16.4 us forward, 58.8 -> 37.4 us
 // with its backward; a 150-token layer 3000 -> 3000, r = 768 66.1 -> 41.1 us; a
 // 2048-token 350M-shaped block 268 -> 192 us.
-//   Z   from K = 1024 on (13 k-blocks with few tiles): shorter ones are no slower
-//       unsplit (forward of 2 to 74 tiles, split against unsplit: 8 k-blocks 1.12 to
-//       1.27, 12 1.04 to 1.21, 13 and 14 0.97 to 1.02 up to 24 tiles and 1.05 to 1.17
-//       above; from 16 on the other way is the slabs', 0.65 to 0.97, and above 48
-//       tokens, or 64 in one tile: with fewer rows their reduce is the shorter way: one
-//       tile of 40 tokens, K = 1024 to 11008 1.05 to 1.11, of 128 tokens 0.88 to
-//       0.95; three tiles of 40 tokens 1.04, of 64 0.94 to 0.96).
+//   Z   from K = 1024 on (13 k-blocks with few tiles, 12 where the last is not whole):
+//       shorter ones are no slower unsplit (forward of 2 to 74 tiles, split against
+//       unsplit: 8 k-blocks 1.12 to 1.27, 12 1.04 to 1.21, but K = 712 0.92 to 0.98 up
+//       to 24 tiles, 13 and 14 0.97 to 1.02 up to 24 and 1.05 to 1.17 above; from 16 on
+//       the other way is the slabs', 0.65 to 0.97, and above 48 tokens, or 64 in one
+//       tile: with fewer rows their reduce is the shorter way: one tile of 40 tokens, K =
+//       1024 to 11008 1.05 to 1.11, of 128 tokens 0.88 to 0.95; three tiles of 40 tokens
+//       1.04, of 64 0.94 to 0.96).
 //   dZ  where the split takes enough k-blocks off the longest CTA to pay for the
 //       exchange (whole backward, split against unsplit: 5 fewer 1.00 to 1.04, 8
 //       0.93 to 1.03; in two splits, whose SMs the unsplit tiles half fill, 8 fewer
@@ -342,7 +343,8 @@ int rank_gemm_splits(int64_t n, int64_t N, int64_t K, int count, int sigma, int 
     if (2 * tiles > sms) return 1;
     const int kb = static_cast<int>((K + BK - 1) / BK);
     const bool cheap = sigma != SIG_GELU;
-    if (cheap && !dz && (kb < 16 ? kb < 13 || tiles > 24 : n <= (tiles == 1 ? 64 : 48))) return 1;
+    const bool few_kb = kb < (K % BK == 0 ? 13 : 12);
+    if (cheap && !dz && (kb < 16 ? few_kb || tiles > 24 : n <= (tiles == 1 ? 64 : 48))) return 1;
     const int S = cluster_splits(static_cast<int>(tiles), kb, sms);
     const int least = cheap ? (S == 2 ? 9 : 8) : (tiles >= 48 ? 5 : 0);   // k-blocks saved
     if (dz && n > THIN_MAX_TOKENS && kb - (kb + S - 1) / S < least) return 1;
