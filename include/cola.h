@@ -124,13 +124,15 @@ cola_status_t cola_workspace_init(void* ws, void* stream);
  *                   and INFER (H is then formed in the workspace and not kept).
  * Two tensor-core GEMMs: Z/H (sigma fused in the epilogue), then Y.  With few
  * output tiles their K ranges are split over thread-block clusters that add the
- * partials on chip (cola_set_cluster_splitk; always with at most 32 tokens, or
- * 64 at r >= 256).  For r = 64 or 128 when both products are HBM-bound (neither
+ * partials on chip: Z/H where that is the faster way (cola_set_cluster_splitk),
+ * and, whatever that is set to, Z/H of at most 32 tokens (64 at r >= 256) and Y of
+ * at most 32 (48 at r >= 512, 64 at r >= 1024; the gated product with few tiles),
+ * but for a layer that has the single-kernel form.  For r = 64 or 128 when both products are HBM-bound (neither
  * compute-heavy nor, at d_in >= 1024, of fewer tiles than half the SMs) and n is
  * at most 128 tokens per SM (19456 on GB300), one kernel instead: each CTA keeps
  * the H of its 128-row tile in shared memory between the two products (H is an
  * intermediate of Eq. (main-fwd), not an output), storing Z and H only as the
- * mode saves them; the results are the same bit for bit
+ * mode saves them; the results are the same bit for bit as its two GEMMs unsplit
  * (cola_set_fused_forward).  Large GEMMs whose A has rows that do not begin on
  * 32-byte sectors (ld_a % 16 != 0) first copy it to an aligned pitch in the
  * workspace, where it has room (dX too). */
@@ -435,15 +437,17 @@ cola_status_t cola_set_fused_backward(int32_t enable);
 
 /* Launches of few output tiles split their K range to fill the SMs: the weight
  * gradients with a short token walk (a few thousand tokens), and the rank-r
- * products Z = X A^T and dZ = dY B of up to a few thousand tokens.  1
+ * products Z = X A^T and dZ = dY B of up to a few thousand tokens, where K is long
+ * enough (or sigma costly enough) for the split to pay.  1
  * (default): the splits of a 128 x 128 tile run as one thread-block cluster of
  * up to 8 CTAs that adds the partial tiles on chip, in a fixed order, and
  * applies the epilogue in the same launch; 0: weight gradients and Z/H with
  * fp32 partials in the workspace and a reduce launch, dZ unsplit.  The two add
  * the same partials in the same order only when they split alike, so results
  * may differ in the last bits between the settings (each is deterministic run
- * to run).  The forward GEMMs of at most 32 tokens (64 at r >= 256) always
- * reduce in clusters.  How many ways a tile is split depends on how many
+ * to run).  The forward GEMMs of few tokens reduce in clusters either way
+ * (cola_fwd), except those of a layer that has the single-kernel form, which runs
+ * that kernel or, with it switched off, two unsplit GEMMs.  How many ways a tile is split depends on how many
  * clusters the device runs at once.  enable outside {0, 1}: COLA_ERR_INVALID. */
 cola_status_t cola_set_cluster_splitk(int32_t enable);
 

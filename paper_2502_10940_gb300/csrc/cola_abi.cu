@@ -355,7 +355,8 @@ cola_status_t run_cluster_wgrad(int count, const CredJob* jobs, int64_t ntok, in
 // reduce launch.  Its 4-stage, one-tile-per-CTA form is made for short token
 // walks: at 65536 tokens (the LLaMA-60M block, 128-171 k-blocks per CTA) it ran
 // the weight gradients 60 -> 93 us.  Walks so short that the most splits leave a
-// CTA at most CLUSTER_SHORT_KPS k-blocks take those, also in two waves.
+// CTA at most CLUSTER_SHORT_KPS k-blocks take those, counted as one wave even where
+// the device runs fewer such clusters at once and a second follows.
 constexpr int CLUSTER_MAX_KPS = 32;
 constexpr int CLUSTER_SHORT_KPS = 8;
 
@@ -968,9 +969,9 @@ cola_status_t run_wgrad(const WgradPlan& w, int64_t ntok, const WgradJob* jobs, 
                         size_t part_bytes, unsigned int* status, int sms, cudaStream_t st)
 {
     {
-        // a small launch: the token splits reduced inside clusters, when one
-        // wave of clusters costs less than the planned schedule with its
-        // reduce launch (counted as REDUCE_LAUNCH_KB k-block steps)
+        // a small launch: the token splits reduced inside clusters, when their
+        // waves cost no more than the planned schedule with its reduce launch
+        // (counted as REDUCE_LAUNCH_KB k-block steps)
         const int Sc = wgrad_cluster_splits(w, ntok, accumulate_f32, sms);
         if (Sc > 1) {
             CredJob J[MAX_GROUP];

@@ -117,16 +117,18 @@ struct GemmParams {
     // step reads each B-operand panel of its tiles once; column-major keeps a
     // wave on few B panels, for problems whose B operand is the larger one.
     int n_major;
-    // The bf16 output behind map_d, for the one 32-column chunk per row block
-    // that holds a ragged right edge (N % 8 != 0): a TMA store clips at
-    // 16-byte granularity and would write the row padding past column N, so
-    // that chunk is stored with masked direct stores instead.
+    // The bf16 output behind map_d, for the one chunk per row block that holds a
+    // ragged right edge (N % 8 != 0): a TMA store clips at 16-byte granularity and
+    // would write the row padding past column N, so that chunk is stored directly,
+    // clipped at N: a staged 64-column box by coalesced rows (EPI_STORE64, plain
+    // outputs of CTA pairs, EPI_GLU), 64 columns a thread's row (the gated dX), or 32
+    // columns element by element (the other epilogues).
     __nv_bfloat16* d_ptr;
     long long d_ld;
     int sigma;
     unsigned int* status;
     // gated MLP: the outputs behind map_d2 (EPI_GLU, EPI_GLU_BWD) and map_d3
-    // (EPI_GLU), for the masked stores of a ragged right edge (pitch d_ld)
+    // (EPI_GLU), for the clipped stores of a ragged right edge (pitch d_ld)
     int glu_half;                 // EPI_GLU: k-blocks of the gate half; the up half reads map_b2
     __nv_bfloat16* d2_ptr;
     __nv_bfloat16* d3_ptr;

@@ -12,7 +12,8 @@
 //     N operand (n rounded up to 16): a tile's fp32 result is 128 x 16..64
 //     instead of the 128 x 128 of a token-major tile that is mostly padding, so
 //     the K splits of a tile, on one thread-block cluster, exchange 8 to 32 KB
-//     per CTA on chip and no reduce launch follows.
+//     per CTA on chip (twice that for the gated product's two halves) and no
+//     reduce launch follows.
 //   - Weights do not depend on the kernel before.  The second GEMM of a call
 //     issues its weight loads before it waits for the first one (programmatic
 //     dependent launch; every kernel of the library lets its successor start
@@ -92,7 +93,7 @@ __host__ __device__ constexpr int thin_ring_bytes(int stages, int NT, bool glu)
 }
 __host__ __device__ constexpr int thin_recv_bytes(int S, int TB, bool glu) { return S > 1 ? S * TB * BM * 4 * (glu ? 2 : 1) : 0; }
 constexpr int THIN_BAR_BYTES = 256;
-constexpr int THIN_SMEM_BUDGET = 110 * 1024;   // two CTAs per SM
+constexpr int THIN_SMEM_BUDGET = 110 * 1024;   // two CTAs per SM (one where the gated product takes more: thin_splits)
 __host__ __device__ constexpr int thin_smem_bytes(int stages, int NT, int S, int TB, bool glu)
 {
     return 1024 + thin_ring_bytes(stages, NT, glu) + thin_recv_bytes(S, TB, glu) + THIN_BAR_BYTES;
